@@ -53,20 +53,20 @@ constexpr int kMaxK = 1024;
 #endif
 
 // Per kernel: a register budget, as 256-thread blocks per SM, where it was
-// measured to pay (the A/B against uncapped builds, GB300).  The one-species
-// birth-death structure's round-to-nearest kernels (not fp64) fit 48
-// registers without spilling: five blocks (40 warps) instead of four, +16%.
-// For Schloegl, telegraph and dimer the same budget costs about 8% more
-// instructions and is slower; 64 registers for mixed stochastic rounding and
-// fp64 (-2%, -4%) and 80 for uniform stochastic rounding (0..+2%) did not pay
-// either.  Every other kernel keeps the compiler's choice.
+// measured to pay.  The one-species birth-death structure's round-to-nearest
+// kernels (not fp64) fit 64 registers: four blocks, 9.6 ms for 10^6
+// trajectories with 101 snapshots (mixed f16) against 10.2 ms at five blocks
+// (48 registers) and 10.0 ms at three.  Everywhere else every budget was slower
+// than the compiler's choice (three / four / five blocks: Schloegl mixed bf16
+// +4 / +6 / +4%, uniform f16 SR +6 / +21 / +27%, telegraph +6 / +5 / +6%,
+// repressilator +4 / +11 / +23%).
 #ifndef SSA_KERNEL_BUDGETS
 #define SSA_KERNEL_BUDGETS 1   // 0: every kernel at SSA_MIN_BLOCKS (for comparisons)
 #endif
 
 template <class Model, int PREC, int SR>
 struct KernelMinBlocks {
-    static constexpr int value = (SSA_KERNEL_BUDGETS && Model::N == 1 && SR == 0 && PREC != 0) ? 5 : SSA_MIN_BLOCKS;
+        static constexpr int value = (SSA_KERNEL_BUDGETS && Model::N == 1 && SR == 0 && PREC != 0) ? 4 : SSA_MIN_BLOCKS;
 };
 
 enum Precision { FP64 = 0, FP32 = 1, MIXED_F16 = 2, MIXED_BF16 = 3, UNIFORM_F16 = 4, UNIFORM_BF16 = 5 };
@@ -1089,14 +1089,46 @@ static __device__ __noinline__ unsigned pool_decide(int *lock, int *count_p, uns
     return (op << 24) | (base << 12) | num;
 }
 
+// A lane's record out of and into the pool.
+template <class Model, int PREC>
+__device__ __forceinline__ void lane_take(const RunArgs &a, const TailPool<Model, PREC> *p, int s, Lane<Model, PREC> &L,
+                                          const typename ModeTraits<PREC>::P *smp)
+{
+    using P = typename ModeTraits<PREC>::P;
+    init_lane<Model, PREC>(a, L, p->item[s], smp);
+    L.n = p->n[s];
+    L.t = p->t[s];
+    L.k = p->k[s];
+    L.status = p->status[s];
+    unroll<Model::N>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        L.x[i] = p->x[i][s];
+    });
+    L.s_next = L.k < a.K ? smp[L.k] : P(__int_as_float(0x7F800000));
+}
+
+template <class Model, int PREC>
+__device__ __forceinline__ void lane_give(const RunArgs &, TailPool<Model, PREC> *p, int s, Lane<Model, PREC> &L)
+{
+    p->item[s] = L.item;
+    p->n[s] = L.n;
+    p->t[s] = L.t;
+    p->k[s] = L.k;
+    p->status[s] = L.status;
+    unroll<Model::N>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        p->x[i][s] = L.x[i];
+    });
+    L.active = false;
+}
+
 // One visit of a warp to its block's pool at a refill check (whole warp).
 // Takes records into idle lanes, or gives the warp's trajectories away.
 // Returns true when the warp leaves the work loop.
-template <class Model, int PREC>
-__device__ __forceinline__ bool pool_visit(const RunArgs &a, TailPool<Model, PREC> *p, Lane<Model, PREC> &L,
+template <class Model, int PREC, class LaneT>
+__device__ __forceinline__ bool pool_visit(const RunArgs &a, TailPool<Model, PREC> *p, LaneT &L,
                                            const typename ModeTraits<PREC>::P *smp)
 {
-    using P = typename ModeTraits<PREC>::P;
     const unsigned lane = threadIdx.x & 31u;
     const int w = (int)(threadIdx.x >> 5);
     const unsigned busy = __ballot_sync(0xFFFFFFFFu, L.active);
@@ -1122,31 +1154,9 @@ __device__ __forceinline__ bool pool_visit(const RunArgs &a, TailPool<Model, PRE
     const unsigned below = (1u << lane) - 1u;
     if (op == 1 && !L.active) {
         const int r = __popc(~busy & below);
-        if (r < num) {
-            const int s = base + r;
-            init_lane<Model, PREC>(a, L, p->item[s], smp);
-            L.n = p->n[s];
-            L.t = p->t[s];
-            L.k = p->k[s];
-            L.status = p->status[s];
-            unroll<Model::N>([&](auto I) {
-                constexpr int i = decltype(I)::value;
-                L.x[i] = p->x[i][s];
-            });
-            L.s_next = L.k < a.K ? smp[L.k] : P(__int_as_float(0x7F800000));
-        }
+        if (r < num) lane_take(a, p, base + r, L, smp);
     } else if (op == 2 && L.active) {
-        const int s = base + __popc(busy & below);
-        p->item[s] = L.item;
-        p->n[s] = L.n;
-        p->t[s] = L.t;
-        p->k[s] = L.k;
-        p->status[s] = L.status;
-        unroll<Model::N>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            p->x[i][s] = L.x[i];
-        });
-        L.active = false;
+        lane_give(a, p, base + __popc(busy & below), L);
     }
     __syncwarp();
     if (lane == 0) {
@@ -1214,10 +1224,29 @@ __device__ __forceinline__ void run_queue(const RunArgs &a, const typename ModeT
     }
 }
 
-template <int PREC>
-__device__ __forceinline__ void load_samples(const double *samples, int K, typename ModeTraits<PREC>::P *smp)
+}  // namespace ssa
+
+#include "ssa_fast.cuh"
+
+namespace ssa {
+
+// Compiled structures run the fast step, everything else the general one.
+template <class Model, int PREC, int SR>
+__device__ __forceinline__ void run_any(const RunArgs &a, const typename ModeTraits<PREC>::P *smp,
+                                        typename ModeTraits<PREC>::P t_end, const double2 *ln2,
+                                        TailPool<Model, PREC> *pool = nullptr)
 {
-    for (int k = threadIdx.x; k < K; k += blockDim.x) smp[k] = to_time<PREC>(samples[k]);
+    if constexpr (std::is_same<Model, GeneralModel>::value) run_queue<Model, PREC, SR>(a, smp, t_end, pool);
+    else run_queue_fast<Model, PREC, SR>(a, smp, t_end, ln2, pool);
+}
+
+template <int PREC>
+__device__ __forceinline__ void load_samples(const double *samples, int K, typename ModeTraits<PREC>::P *smp, double2 *ln2)
+{
+    using P = typename ModeTraits<PREC>::P;
+    if constexpr (PREC == FP64)
+        for (int k = threadIdx.x; k < kLn2Rows; k += blockDim.x) ln2[k] = ln2_row(k);
+    for (int k = threadIdx.x; k < K; k += blockDim.x) smp[k] = to_time<PREC>(samples[k]) + P(0);   // -0 becomes +0
     __syncthreads();
 }
 
@@ -1229,11 +1258,12 @@ __global__ void __launch_bounds__(256, (KernelMinBlocks<Model, PREC, SR>::value)
     using P = typename ModeTraits<PREC>::P;
     __shared__ P smp[kMaxK];
     __shared__ TailPool<Model, PREC> pool;
+    __shared__ double2 ln2[PREC == FP64 ? kLn2Rows : 1];
     const bool pooled = a.tail_stats != nullptr;
     if (pooled) pool_init(&pool);
-    load_samples<PREC>(a.samples, a.K, smp);   // ends with __syncthreads
+    load_samples<PREC>(a.samples, a.K, smp, ln2);   // ends with __syncthreads
     for (int pass = 0;; ++pass) {
-        run_queue<Model, PREC, SR>(a, smp, to_time<PREC>(a.t_end), pooled ? &pool : nullptr);
+        run_any<Model, PREC, SR>(a, smp, to_time<PREC>(a.t_end), ln2, pooled ? &pool : nullptr);
         if (!pooled || pass > 0) break;
         // every warp has left the loop: records stranded by a lock wait that
         // gave up are resumed by warp 0 (the pool no longer changes)
@@ -1274,17 +1304,17 @@ namespace ssa {
 
 template <int FAM, int PREC, int SR>
 __device__ __forceinline__ void run_family(const RunArgs &a, int normalise, const typename ModeTraits<PREC>::P *smp,
-                                           typename ModeTraits<PREC>::P t_end)
+                                           typename ModeTraits<PREC>::P t_end, const double2 *ln2)
 {
-    if constexpr (FAM == 1) run_queue<StaticModel<models::BirthDeath, false>, PREC, SR>(a, smp, t_end);
+    if constexpr (FAM == 1) run_any<StaticModel<models::BirthDeath, false>, PREC, SR>(a, smp, t_end, ln2);
     else if constexpr (FAM == 2) {
-        if (normalise) run_queue<StaticModel<models::Schlogl, true>, PREC, SR>(a, smp, t_end);
-        else run_queue<StaticModel<models::Schlogl, false>, PREC, SR>(a, smp, t_end);
+        if (normalise) run_any<StaticModel<models::Schlogl, true>, PREC, SR>(a, smp, t_end, ln2);
+        else run_any<StaticModel<models::Schlogl, false>, PREC, SR>(a, smp, t_end, ln2);
     }
-    else if constexpr (FAM == 3) run_queue<StaticModel<models::Telegraph, false>, PREC, SR>(a, smp, t_end);
-    else if constexpr (FAM == 4) run_queue<StaticModel<models::Dimer, false>, PREC, SR>(a, smp, t_end);
-    else if constexpr (FAM == 5) run_queue<StaticModel<models::Repressilator, false>, PREC, SR>(a, smp, t_end);
-    else run_queue<GeneralModel, PREC, SR>(a, smp, t_end);
+    else if constexpr (FAM == 3) run_any<StaticModel<models::Telegraph, false>, PREC, SR>(a, smp, t_end, ln2);
+    else if constexpr (FAM == 4) run_any<StaticModel<models::Dimer, false>, PREC, SR>(a, smp, t_end, ln2);
+    else if constexpr (FAM == 5) run_any<StaticModel<models::Repressilator, false>, PREC, SR>(a, smp, t_end, ln2);
+    else run_any<GeneralModel, PREC, SR>(a, smp, t_end, ln2);
 }
 
 // FAMS lists the structure families compiled into this instantiation; a
@@ -1294,12 +1324,13 @@ __global__ void __launch_bounds__(256) ssa_batch_kernel(const __grid_constant__ 
 {
     using P = typename ModeTraits<PREC>::P;
     __shared__ P smp[kMaxK];
-    load_samples<PREC>(b.samples, b.K, smp);
+    __shared__ double2 ln2[PREC == FP64 ? kLn2Rows : 1];
+    load_samples<PREC>(b.samples, b.K, smp, ln2);
     const P t_end = to_time<PREC>(b.t_end);
     for (int g = 0; g < b.n_groups; ++g) {
         const RunArgs &a = b.groups[g];
         const int fam = b.family[g];
-        ((fam == FAMS ? (run_family<FAMS, PREC, SR>(a, b.normalise, smp, t_end), 0) : 0), ...);
+        ((fam == FAMS ? (run_family<FAMS, PREC, SR>(a, b.normalise, smp, t_end, ln2), 0) : 0), ...);
     }
 }
 
