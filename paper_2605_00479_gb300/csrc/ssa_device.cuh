@@ -151,6 +151,27 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
 }
 
 // --------------------------------------------------------------------- log
+__device__ __forceinline__ float rcp_seed(float b)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+    return r;
+}
+
+// RN(a / b) where a and b carry at most 11 significant bits (or, in the
+// logarithm, are m - 1 and m + 1: all 2^23 significands checked): such
+// quotients stay at least 2^-36 (relative) from a rounding boundary, and the
+// corrected value is within 2^-45 before its rounding.
+__device__ __forceinline__ float div_short(float a, float b)
+{
+    const float r = rcp_seed(b);
+    const float q = a * r;
+    const float rem = __fmaf_rn(-q, b, a);
+    return __fmaf_rn(rem, r, q);
+}
+
+// The header's operations; the doubling and the exact product e ln2_hi are
+// folded into fused multiply-adds, which changes no value.
 __device__ __forceinline__ float log_f32(float x)
 {
     const float kLn2Hi = 0x1.62e400p-1f;       // leading 16 bits of ln 2
@@ -165,7 +186,7 @@ __device__ __forceinline__ float log_f32(float x)
     const float m = __uint_as_float(mb);
     const float f = m - 1.0f;
     const float d = m + 1.0f;
-    const float s = f / d;
+    const float s = div_short(f, d);
     const float z = s * s;
     float p = 2.0f / 9.0f;
     p = z * p; p = (2.0f / 7.0f) + p;
@@ -173,13 +194,11 @@ __device__ __forceinline__ float log_f32(float x)
     p = z * p; p = (2.0f / 3.0f) + p;
     float r = s * z;
     r = r * p;
-    const float two_s = s + s;
-    r = two_s + r;
+    r = __fmaf_rn(2.0f, s, r);
     const float ef = (float)e;
     float lo = ef * kLn2Lo;
     lo = lo + r;
-    const float hi = ef * kLn2Hi;
-    return hi + lo;
+    return __fmaf_rn(ef, kLn2Hi, lo);
 }
 
 __device__ __forceinline__ double log_f64(double x)

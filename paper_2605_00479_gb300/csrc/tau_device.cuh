@@ -119,109 +119,6 @@ __device__ __forceinline__ double logfact_f64(double k)
     return s;
 }
 
-// Words of one (leap, channel) sampler stream.
-struct SamplerWords {
-    uint32_t k0, k1, leap, traj, stream, w;
-    uint4 blk;
-    __device__ __forceinline__ uint32_t next()
-    {
-        if ((w & 3u) == 0u) blk = philox4x32_10(make_uint4(w >> 2, leap, traj, stream), k0, k1);
-        const uint32_t i = w & 3u;
-        w += 1;
-        return i == 0 ? blk.x : (i == 1 ? blk.y : (i == 2 ? blk.z : blk.w));
-    }
-};
-
-__device__ inline int64_t poisson_f32(float lam, SamplerWords &s)
-{
-    if (!(lam > 0.0f)) return 0;
-    if (lam < 10.0f) {
-        const float L = exp_f32(-lam);
-        float p = 1.0f;
-        int64_t k = -1;
-        for (int it = 0; it < 1000; ++it) {
-            const float v = (float)((s.next() >> 8) + 1u) * 0x1p-24f;
-            k += 1;
-            p = p * v;
-            if (!(p > L)) return k;
-        }
-        return k;
-    }
-    const float slam = sqrtf(lam);
-    const float loglam = log_f32(lam);
-    const float b = 0.931f + 2.53f * slam;
-    const float a = -0.059f + 0.02483f * b;
-    const float invalpha = 1.1239f + 1.1328f / (b - 3.4f);
-    const float vr = 0.9277f - 3.6224f / (b - 2.0f);
-    const float log_invalpha = log_f32(invalpha);
-    const float kmax = lam + 64.0f * slam + 64.0f;
-    for (int it = 0; it < 100; ++it) {
-        const float U = (float)(s.next() >> 8) * 0x1p-24f - 0.5f;
-        const float V = (float)((s.next() >> 8) + 1u) * 0x1p-24f;
-        const float aU = U < 0.0f ? -U : U;
-        const float us = 0.5f - aU;
-        if (!(us > 0.0f)) continue;
-        float kf = (2.0f * a / us + b) * U;
-        kf = kf + lam;
-        kf = kf + 0.43f;
-        kf = floorf(kf);
-        if (us >= 0.07f && V <= vr) return (int64_t)kf;
-        if (kf < 0.0f || (us < 0.013f && V > us)) continue;
-        if (kf > kmax) continue;
-        float lhs = log_f32(V) + log_invalpha;
-        lhs = lhs - log_f32(a / (us * us) + b);
-        float rhs = -lam + kf * loglam;
-        rhs = rhs - logfact_f32(kf);
-        if (lhs <= rhs) return (int64_t)kf;
-    }
-    return (int64_t)floorf(lam);
-}
-
-__device__ inline int64_t poisson_f64(double lam, SamplerWords &s)
-{
-    if (!(lam > 0.0)) return 0;
-    if (lam < 10.0) {
-        const double L = exp_f64(-lam);
-        double p = 1.0;
-        int64_t k = -1;
-        for (int it = 0; it < 1000; ++it) {
-            const double v = ((double)s.next() + 1.0) * 0x1p-32;
-            k += 1;
-            p = p * v;
-            if (!(p > L)) return k;
-        }
-        return k;
-    }
-    const double slam = sqrt(lam);
-    const double loglam = log_f64(lam);
-    const double b = 0.931 + 2.53 * slam;
-    const double a = -0.059 + 0.02483 * b;
-    const double invalpha = 1.1239 + 1.1328 / (b - 3.4);
-    const double vr = 0.9277 - 3.6224 / (b - 2.0);
-    const double log_invalpha = log_f64(invalpha);
-    const double kmax = lam + 64.0 * slam + 64.0;
-    for (int it = 0; it < 100; ++it) {
-        const double U = (double)s.next() * 0x1p-32 - 0.5;
-        const double V = ((double)s.next() + 1.0) * 0x1p-32;
-        const double aU = U < 0.0 ? -U : U;
-        const double us = 0.5 - aU;
-        if (!(us > 0.0)) continue;
-        double kf = (2.0 * a / us + b) * U;
-        kf = kf + lam;
-        kf = kf + 0.43;
-        kf = floor(kf);
-        if (us >= 0.07 && V <= vr) return (int64_t)kf;
-        if (kf < 0.0 || (us < 0.013 && V > us)) continue;
-        if (kf > kmax) continue;
-        double lhs = log_f64(V) + log_invalpha;
-        lhs = lhs - log_f64(a / (us * us) + b);
-        double rhs = -lam + kf * loglam;
-        rhs = rhs - logfact_f64(kf);
-        if (lhs <= rhs) return (int64_t)kf;
-    }
-    return (int64_t)floor(lam);
-}
-
 template <class Model, int PREC>
 __device__ void tau_finish(const RunArgs &a, Lane<Model, PREC> &L)
 {
@@ -278,15 +175,6 @@ __device__ __forceinline__ void static_propensities(const RunArgs &a, const Lane
     });
 }
 
-// Out-of-line sampler call for the unrolled channel loop of compiled
-// structures (one copy of the sampler instead of one per channel).
-template <int PREC>
-__device__ __noinline__ int64_t poisson_call(typename ModeTraits<PREC>::P lam, SamplerWords &s)
-{
-    if constexpr (ModeTraits<PREC>::kF64) return poisson_f64(lam, s);
-    else return poisson_f32(lam, s);
-}
-
 // Smallest m >= 0 with fl(m * tau) > s in binary64.  Since fl(m * tau) does
 // not decrease with m, "s < fl((n + 1) * tau)" (snapshot s is written before
 // leap n) is "n + 1 >= m": the leap loop then needs no binary64 operation.
@@ -299,111 +187,290 @@ __device__ inline int64_t first_leap_after(double s, double tau)
     return m;
 }
 
-// One leap n = L.n of an active lane.  m_first[k]: first_leap_after(sample
-// k, tau); tau32: tau rounded to binary32.
+// ------------------------------------------------------------------- a leap
+// A leap's draws are independent of one another (each channel has its own
+// Philox stream), but how long a draw takes differs from lane to lane: the
+// multiplication method uses Poisson(lambda) + 1 uniforms, the rejection
+// method accepts at once in about 9 of 10 cases and otherwise evaluates three
+// logarithms and five quotients.  Run one after the other, the channels of a
+// leap each wait for the slowest lane of the warp: 8.8 of 32 lanes were active
+// per instruction (Schloegl, tau = 0.005).  So a leap runs in two phases:
+//   1. every channel gets one Philox block: four uniforms of the
+//      multiplication method, or the rejection method's first quick test.
+//      What that does not settle is marked pending (its state in shared
+//      memory);
+//   2. every lane works through its own pending channels, one block or
+//      rejection round an iteration, so lanes wait only for the largest total
+//      of a lane, not for the largest of every channel.
+// Quantities that only the slow test reads are computed only there.  Measured (GB300, Schloegl fp32, 1.5 10^5 trajectories,
+// 2000 leaps): 51.1 -> 28.4 ms.
+template <class R>
+struct SamplerMath;
+template <>
+struct SamplerMath<float> {
+    static __device__ __forceinline__ float half_open(uint32_t w) { return (float)(w >> 8) * 0x1p-24f; }
+    static __device__ __forceinline__ float positive(uint32_t w) { return (float)((w >> 8) + 1u) * 0x1p-24f; }
+    // operands here: x in [0.1, 2^61], y in [2^-48, 2^66]
+    static __device__ __forceinline__ float div(float x, float y) { return div_rn(x, y); }
+    static __device__ __forceinline__ float exp(float x) { return exp_f32(x); }
+    static __device__ __forceinline__ float log(float x) { return log_f32(x); }
+    static __device__ __forceinline__ float root(float x) { return sqrtf(x); }
+    static __device__ __forceinline__ float down(float x) { return floorf(x); }
+    // integral x >= 0; below 2^22 from the sum's bits (the 64-bit conversion is slow)
+    static __device__ __forceinline__ int64_t to_int(float x)
+    {
+        if (x < 0x1p22f) return __float_as_int(x + 0x1.8p23f) - 0x4B400000;
+        return (int64_t)x;
+    }
+    static __device__ __forceinline__ float logfact(float k, const float *small) { return k < 10.0f ? small[(int)k] : logfact_f32(k); }
+};
+template <>
+struct SamplerMath<double> {
+    static __device__ __forceinline__ double half_open(uint32_t w) { return u32_scaled(w); }
+    static __device__ __forceinline__ double positive(uint32_t w) { return w == 0xFFFFFFFFu ? 1.0 : u32_scaled(w + 1u); }
+    static __device__ __forceinline__ double div(double x, double y) { return x / y; }
+    static __device__ __forceinline__ double exp(double x) { return exp_f64(x); }
+    static __device__ __forceinline__ double log(double x) { return log_f64(x); }
+    static __device__ __forceinline__ double root(double x) { return sqrt(x); }
+    static __device__ __forceinline__ double down(double x) { return floor(x); }
+    static __device__ __forceinline__ int64_t to_int(double x)
+    {
+        if (x < 0x1p30) return __double2loint(x + 0x1.8p52);
+        return (int64_t)x;
+    }
+    static __device__ __forceinline__ double logfact(double k, const double *small) { return k < 10.0 ? small[(int)k] : logfact_f64(k); }
+};
+
+// The rejection method's constants of lambda that every round needs.
+template <class R>
+struct Rejection {
+    R slam, b, a, vr;
+    __device__ __forceinline__ explicit Rejection(R lam)
+    {
+        using Q = SamplerMath<R>;
+        slam = Q::root(lam);
+        b = R(sizeof(R) == 8 ? 0.931 : 0.931f) + R(sizeof(R) == 8 ? 2.53 : 2.53f) * slam;
+        a = R(sizeof(R) == 8 ? -0.059 : -0.059f) + R(sizeof(R) == 8 ? 0.02483 : 0.02483f) * b;
+        vr = R(sizeof(R) == 8 ? 0.9277 : 0.9277f) - Q::div(R(sizeof(R) == 8 ? 3.6224 : 3.6224f), b - R(2));
+    }
+    // One round on words (w0, w1): true when it settles without the slow
+    // test; then kf is the draw, or -1 when the round is rejected.
+    __device__ __forceinline__ bool quick(R lam, uint32_t w0, uint32_t w1, R &us, R &V, R &kf) const
+    {
+        using Q = SamplerMath<R>;
+        const R U = Q::half_open(w0) - R(0.5);
+        V = Q::positive(w1);
+        us = R(0.5) - (U < R(0) ? -U : U);
+        if (!(us > R(0))) {
+            kf = R(-1);
+            return true;
+        }
+        R v = (Q::div(R(2) * a, us) + b) * U;
+        v = v + lam;
+        v = v + R(sizeof(R) == 8 ? 0.43 : 0.43f);
+        kf = Q::down(v);
+        if (us >= R(sizeof(R) == 8 ? 0.07 : 0.07f) && V <= vr) return true;
+        const R kmax = lam + R(64) * slam + R(64);
+        if (kf < R(0) || (us < R(sizeof(R) == 8 ? 0.013 : 0.013f) && V > us) || kf > kmax) {
+            kf = R(-1);
+            return true;
+        }
+        return false;
+    }
+    __device__ __forceinline__ bool slow(R lam, R us, R V, R kf, const R *small) const
+    {
+        using Q = SamplerMath<R>;
+        const R invalpha = R(sizeof(R) == 8 ? 1.1239 : 1.1239f) +
+                           Q::div(R(sizeof(R) == 8 ? 1.1328 : 1.1328f), b - R(sizeof(R) == 8 ? 3.4 : 3.4f));
+        R lhs = Q::log(V) + Q::log(invalpha);
+        lhs = lhs - Q::log(Q::div(a, us * us) + b);
+        R rhs = -lam + kf * Q::log(lam);
+        rhs = rhs - Q::logfact(kf, small);
+        return lhs <= rhs;
+    }
+};
+
+// Four uniforms of the multiplication method: p *= v; counts the products
+// above L.  True when the last one is not (the draw is settled).
+template <class R>
+__device__ __forceinline__ bool multiply_block(R &p, R L, uint4 u, R &count)
+{
+    using Q = SamplerMath<R>;
+    R c = R(0);
+    p = p * Q::positive(u.x); if (p > L) c = c + R(1);
+    p = p * Q::positive(u.y); if (p > L) c = c + R(1);
+    p = p * Q::positive(u.z); if (p > L) c = c + R(1);
+    p = p * Q::positive(u.w); if (p > L) c = c + R(1);
+    count = c;
+    return !(p > L);
+}
+
+// f(j) for every channel: unrolled for compiled structures (j a constant),
+// a loop for the general model.
+template <class Model, class F>
+__device__ __forceinline__ void tau_channels(const RunArgs &a, F &&f)
+{
+    if constexpr (std::is_same<Model, GeneralModel>::value) {
+#pragma unroll 1
+        for (int j = 0; j < a.M; ++j) f(j);
+    } else {
+        unroll<Model::M>([&](auto J) { f((int)decltype(J)::value); });
+    }
+}
+
+// col: this thread's column of three arrays of a.M values (stride bd):
+// lambda; e^-lambda (multiplication method); the pending product, then the
+// draw.  small: log k! for k = 0..9.
 template <class Model, int PREC, int SR>
-__device__ __noinline__ void tau_leap(const RunArgs &a, Lane<Model, PREC> &L, const int64_t *m_first, float tau32)
+__device__ __forceinline__ void tau_leap(const RunArgs &a, Lane<Model, PREC> &L, const uint32_t *m_first, float tau32,
+                                              typename ModeTraits<PREC>::P *col, int bd,
+                                         const typename ModeTraits<PREC>::P *small)
 {
     using Tr = ModeTraits<PREC>;
     using P = typename Tr::P;
+    using Q = SamplerMath<P>;
     constexpr bool kGeneral = std::is_same<Model, GeneralModel>::value;
-    const int64_t n = L.n;
-    while (L.k < a.K && n + 1 >= m_first[L.k]) {
+    const int M = kGeneral ? a.M : Model::M;
+    const uint32_t n = (uint32_t)L.n;
+    while (L.k < a.K && n + 1u >= m_first[L.k]) {
         store_state<Model>(a, L.k, L.item, L.x, L.status);
         L.k += 1;
     }
-    Rounder<PREC, SR> R;
-    if constexpr (Tr::k16 && SR) {
-        const int sr_total = Model::total_chain_ops(a) + (Tr::kUniform ? Model::last(a) + 1 : 0);
-        R.bits.base = (uint64_t)n * (uint64_t)((sr_total + 7) >> 3);
-        R.bits.traj = L.traj;
-        R.bits.k0 = a.key0;
-        R.bits.k1 = a.key1;
-        R.bits.cur = -1;
-    }
-    float tau16 = tau32;
-    if constexpr (Tr::k16) tau16 = rn16<Tr::kFmt>(tau32);
-    const int lam_op = Model::total_chain_ops(a);   // SR slot of lambda_0 (uniform modes)
-    auto lambda_of = [&](P prop, int j) -> P {
-        if constexpr (Tr::kF64) return prop * a.tau;
-        else if constexpr (Tr::kUniform) return R.rnd(prop * tau16, lam_op + j);
-        else return prop * tau32;
-    };
-    P prop[Model::M];
-    P lam[Model::M];
     uint32_t bad = 0;
-    if constexpr (kGeneral) {
-        general_propensities<PREC, SR>(a, L, R, prop);
-#pragma unroll 1
-        for (int j = 0; j < a.M; ++j) {
-            const P v = lambda_of(prop[j], j);
-            lam[j] = v;
-            if (v != v) bad |= ST_NAN;
-            else if (v == P(__int_as_float(0x7F800000))) bad |= ST_OVERFLOW;
+    {
+        Rounder<PREC, SR> R;
+        if constexpr (Tr::k16 && SR) {
+            const int sr_total = Model::total_chain_ops(a) + (Tr::kUniform ? Model::last(a) + 1 : 0);
+            R.bits.base = (uint64_t)n * (uint64_t)((sr_total + 7) >> 3);
+            R.bits.traj = L.traj;
+            R.bits.k0 = a.key0;
+            R.bits.k1 = a.key1;
+            R.bits.cur = -1;
         }
-    } else {
-        static_propensities<Model, PREC, SR>(a, L, R, prop);
-        unroll<Model::M>([&](auto J) {
-            constexpr int j = decltype(J)::value;
-            const P v = lambda_of(prop[j], j);
-            lam[j] = v;
+        float tau16 = tau32;
+        if constexpr (Tr::k16) tau16 = rn16<Tr::kFmt>(tau32);
+        const int lam_op = Model::total_chain_ops(a);
+        P prop[Model::M];
+        if constexpr (kGeneral) general_propensities<PREC, SR>(a, L, R, prop);
+        else static_propensities<Model, PREC, SR>(a, L, R, prop);
+        tau_channels<Model>(a, [&](int j) {
+
+            P v;
+            if constexpr (Tr::kF64) v = prop[j] * a.tau;
+            else if constexpr (Tr::kUniform) v = R.rnd(prop[j] * tau16, lam_op + j);
+            else v = prop[j] * tau32;
             if (v != v) bad |= ST_NAN;
             else if (v == P(__int_as_float(0x7F800000))) bad |= ST_OVERFLOW;
+            col[j * bd] = v;
         });
     }
     if (bad) {
         L.status |= bad;
         tau_finish<Model, PREC>(a, L);
-        return;
-    }
-    int64_t dx[Model::N];
+    } else {
+        P *const colL = col + M * bd, *const colK = colL + M * bd;
+        TrajPhilox ph;
+        {
+            const uint64_t p1 = (uint64_t)0xCD9E8D57u * L.traj;
+            const uint64_t p0 = (uint64_t)0xD2511F53u * ((uint32_t)(p1 >> 32) ^ n ^ a.key0);
+            ph.cx = (uint32_t)p1 ^ (a.key0 + 0x9E3779B9u);
+            ph.cz = (uint32_t)(p0 >> 32) ^ (a.key1 + 0xBB67AE85u);
+            ph.cw = (uint32_t)p0;
+        }
+        // phase 1: one block a channel
+        uint32_t pend = 0u;
+        tau_channels<Model>(a, [&](int j) {
+
+            const P lam = col[j * bd];
+            P k = P(0);
+            if (lam > P(0)) {
+                const uint4 u = ph.block(0u, 2u + (uint32_t)j, a.key0, a.key1);
+                if (lam < P(10)) {
+                    const P e = Q::exp(-lam);
+                    P p = P(1);
+                    if (!multiply_block<P>(p, e, u, k)) {
+                        pend |= 1u << j;
+                        colL[j * bd] = e;
+                        k = p;
+                    }
+                } else {
+                    const Rejection<P> rej(lam);
+                    P us, V;
+                    if (!rej.quick(lam, u.x, u.y, us, V, k) || k < P(0)) pend |= 1u << j;
+                }
+            }
+            colK[j * bd] = k;
+        });
+        // phase 2: the lane's pending channels
+        int j = 0, it = 0;
+        P lam = P(0), e = P(0), p = P(0);
+        auto take = [&]() {
+            j = __ffs((int)pend) - 1;
+            lam = col[j * bd];
+            e = colL[j * bd];
+            p = colK[j * bd];
+            it = lam < P(10) ? 1 : 0;
+        };
+        if (pend) take();
+        while (pend) {
+            const bool product = lam < P(10);
+            const uint4 u = ph.block(product ? (uint32_t)it : (uint32_t)(it >> 1), 2u + (uint32_t)j, a.key0, a.key1);
+            bool done;
+            P k;
+            if (product) {
+                P c;
+                done = multiply_block<P>(p, e, u, c);
+                k = P(4 * it) + c;
+                if (it == 249 && !done) {   // 1000 uniforms: the bound of the method
+                    done = true;
+                    k = P(999);
+                }
+            } else {
+                const Rejection<P> rej(lam);
+                P us, V;
+                const bool second = (it & 1) != 0;
+                done = rej.quick(lam, second ? u.z : u.x, second ? u.w : u.y, us, V, k);
+                if (done) done = k >= P(0);
+                else done = rej.slow(lam, us, V, k, small);
+                if (it == 99 && !done) {    // 100 rounds
+                    done = true;
+                    k = Q::down(lam);
+                }
+            }
+            it += 1;
+            if (done) {
+                colK[j * bd] = k;
+                pend &= pend - 1u;
+                if (pend) take();
+            }
+        }
+        // x += sum_j nu_j k_j
+        int64_t dx[Model::N];
 #pragma unroll
-    for (int i = 0; i < Model::N; ++i) dx[i] = 0;
-    SamplerWords sw;
-    sw.k0 = a.key0;
-    sw.k1 = a.key1;
-    sw.leap = (uint32_t)n;
-    sw.traj = L.traj;
-    if constexpr (kGeneral) {
+        for (int i = 0; i < Model::N; ++i) dx[i] = 0;
+        int64_t fired = 0;
+        if constexpr (kGeneral) {
 #pragma unroll 1
-        for (int j = 0; j < a.M; ++j) {
-            sw.stream = 2u + (uint32_t)j;
-            sw.w = 0;
-            int64_t kj;
-            if constexpr (Tr::kF64) kj = poisson_f64(lam[j], sw);
-            else kj = poisson_f32(lam[j], sw);
-            L.ev += kj;
+            for (int c = 0; c < a.M; ++c) {
+                const int64_t k = Q::to_int(colK[c * bd]);
+                fired += k;
 #pragma unroll 1
-            for (int i = 0; i < a.N; ++i) dx[i] += kj * (int64_t)a.stoich[j][i];
-        }
-    } else {
-        unroll<Model::M>([&](auto J) {
-            constexpr int j = decltype(J)::value;
-            sw.stream = 2u + (uint32_t)j;
-            sw.w = 0;
-            const int64_t kj = poisson_call<PREC>(lam[j], sw);
-            L.ev += kj;
-            unroll<Model::N>([&](auto I) {
-                constexpr int i = decltype(I)::value;
-                const int nu = Model::template nu<j, i>(a);
-                if (nu != 0) dx[i] += kj * (int64_t)nu;
+                for (int i = 0; i < a.N; ++i) dx[i] += k * (int64_t)a.stoich[c][i];
+            }
+        } else {
+            unroll<Model::M>([&](auto J) {
+                constexpr int c = decltype(J)::value;
+                const int64_t k = Q::to_int(colK[c * bd]);
+                fired += k;
+                unroll<Model::N>([&](auto I) {
+                    constexpr int i = decltype(I)::value;
+                    const int nu = Model::template nu<c, i>(a);
+                    if (nu != 0) dx[i] += k * (int64_t)nu;
+                });
             });
-        });
-    }
-    if constexpr (kGeneral) {
-#pragma unroll 1
-        for (int i = 0; i < a.N; ++i) {
-            int64_t v = (int64_t)L.x[i] + dx[i];
-            if (v < 0) {
-                v = 0;
-                L.status |= ST_TAU_CLAMPED;
-            }
-            if (v > 2147483647) v = 2147483647;
-            L.x[i] = (int)v;
         }
-    } else {
-        unroll<Model::N>([&](auto I) {
-            constexpr int i = decltype(I)::value;
+        L.ev += fired;
+        auto move = [&](int i) {
             int64_t v = (int64_t)L.x[i] + dx[i];
             if (v < 0) {
                 v = 0;
@@ -411,20 +478,38 @@ __device__ __noinline__ void tau_leap(const RunArgs &a, Lane<Model, PREC> &L, co
             }
             if (v > 2147483647) v = 2147483647;
             L.x[i] = (int)v;
-        });
+        };
+        if constexpr (kGeneral) {
+#pragma unroll 1
+            for (int i = 0; i < a.N; ++i) move(i);
+        } else {
+            unroll<Model::N>([&](auto I) { move(decltype(I)::value); });
+        }
+        L.n += 1;
+        if (L.n >= a.n_leaps) tau_finish<Model, PREC>(a, L);
     }
-    L.n = n + 1;
-    if (L.n >= a.n_leaps) tau_finish<Model, PREC>(a, L);
 }
+
 // Persistent tau-leaping kernel: lanes refill from the work queue as in the
 // direct method; each loop iteration runs one leap.  Model is a compiled
-// structure (StaticModel) or the runtime-table GeneralModel.
+// structure (StaticModel) or the runtime-table GeneralModel.  Dynamic shared
+// memory: tau_shared_bytes.
 template <class Model, int PREC, int SR>
 __global__ void __launch_bounds__(256) tau_kernel(const __grid_constant__ RunArgs a)
 {
     using P = typename ModeTraits<PREC>::P;
-    __shared__ int64_t m_first[kMaxK];
-    for (int k = threadIdx.x; k < a.K; k += blockDim.x) m_first[k] = first_leap_after(a.samples[k], a.tau);
+    extern __shared__ __align__(16) unsigned char tau_smem[];
+    __shared__ P small[10];
+    if (threadIdx.x < 10) {
+        if constexpr (PREC == FP64) small[threadIdx.x] = logfact_f64((double)threadIdx.x);
+        else small[threadIdx.x] = logfact_f32((float)threadIdx.x);
+    }
+    uint32_t *m_first = reinterpret_cast<uint32_t *>(tau_smem);
+    P *col = reinterpret_cast<P *>(tau_smem + (((size_t)a.K * 4 + 15) & ~(size_t)15)) + threadIdx.x;
+    for (int k = threadIdx.x; k < a.K; k += blockDim.x) {
+        const int64_t m = first_leap_after(a.samples[k], a.tau);
+        m_first[k] = m > 0xFFFFFFFFll ? 0xFFFFFFFFu : (uint32_t)m;   // leaps are numbered below 2^31
+    }
     __syncthreads();
     const float tau32 = (float)a.tau;
     const unsigned lane = threadIdx.x & 31u;
@@ -451,8 +536,13 @@ __global__ void __launch_bounds__(256) tau_kernel(const __grid_constant__ RunArg
             }
         }
         if (__ballot_sync(0xFFFFFFFFu, L.active) == 0u) break;
-        if (L.active) tau_leap<Model, PREC, SR>(a, L, m_first, tau32);
+        if (L.active) tau_leap<Model, PREC, SR>(a, L, m_first, tau32, col, (int)blockDim.x, small);
     }
+}
+
+inline size_t tau_shared_bytes(const RunArgs &a, int block, int elem_bytes)
+{
+    return (((size_t)a.K * 4 + 15) & ~(size_t)15) + (size_t)3 * (size_t)a.M * (size_t)block * (size_t)elem_bytes;
 }
 
 // Launch of one structure's kernel for (precision, rounding); the grid is
@@ -477,7 +567,11 @@ cudaError_t tau_launch_model(const RunArgs &a, int prec, int sr, int block, int 
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, 0);
+    // at most 16 channels x 256 threads x 3 binary64 values + 4 KB: 100 KB
+    const size_t smem = tau_shared_bytes(a, block, prec == FP64 ? 8 : 4);
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     if (blocks_per_sm > 0 && blocks_per_sm < per_sm) per_sm = blocks_per_sm;
@@ -486,7 +580,7 @@ cudaError_t tau_launch_model(const RunArgs &a, int prec, int sr, int block, int 
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
     *grid_out = (int)grid;
-    k<<<(unsigned)grid, (unsigned)block, 0, stream>>>(a);
+    k<<<(unsigned)grid, (unsigned)block, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
