@@ -273,9 +273,10 @@ int ssa_rdme_run(const ssa_model *model, int nx, int ny, int nz, const double *d
  *                      finished lanes to refill, 1..64
  * threads_per_block = 0 restores the library's defaults (the other arguments
  * are then ignored): for single-queue direct-method runs 32 step pairs per
- * check and, per kernel, 256 threads per block unless that keeps fewer than
- * 85% of the resident warps 128-thread blocks would (then 128); (128, 0, 16)
- * for tau-leaping, RDME and batches.  These were the fastest measured.  Once a shape is set, every kind of run uses it.  Tau-leaping and
+ * check and 256 threads per block, 128 where 256 would keep fewer than three
+ * quarters of the resident warps, or 128 or 64 where a run of at most 384
+ * trajectories per SM spreads better over the SMs; (128, 0, 16) for
+ * tau-leaping, RDME and batches.  These were the fastest measured.  Once a shape is set, every kind of run uses it.  Tau-leaping and
  * RDME kernels take only the block size and check for refills after every
  * step.
  * Results never depend on the launch shape; only speed does.  Not

@@ -79,6 +79,28 @@ int rdme_block_size(const RdmeArgs &A, int elem_bytes, bool epochs, int max_bloc
 cudaError_t launch_rdme(const RdmeArgs &A, int family, int norm, int prec, int sr, LaunchConfig cfg,
                         cudaStream_t stream, int *grid_out, int *block_out);
 
+// Threads per block of a direct-method run of n trajectories, when none is set.
+//  * Full GPU: 256 threads -- eight warps hand trajectories to each other at
+//    the end of the launch -- unless that keeps fewer than three quarters of
+//    the warps 128-thread blocks would (Schloegl uniform f16 SR, 16 of 20 warps
+//    a multiprocessor: 256 threads 40.4 against 48.1 ms at 1.5 10^5
+//    trajectories, 176.9 against 179.4 ms at 10^6).
+//  * Up to 384 lanes per multiprocessor the blocks are one wave and latency
+//    counts: the fullest multiprocessor sets the time, so the block shrinks
+//    where that spreads the lanes better (repressilator 5 10^4: 16.5 -> 14.2 ms
+//    with 128 threads; Schloegl fp64 4 10^4: 21.6 -> 17.7 ms, 10^3..2 10^4 mixed
+//    bf16 3.0 -> 2.9 ms with 64).  Above, packing is worth more (Schloegl mixed
+//    bf16 8 10^4: 4.25 ms with 256 threads, 4.33 with 128, 4.73 with 64).
+inline int default_block(long long n, int sms, int p256, int p128)
+{
+    if (n > 384ll * sms) return p256 * 8 * 4 >= p128 * 4 * 3 ? 256 : 128;
+    auto fullest = [&](int b) { return ((n + b - 1) / b + sms - 1) / sms * b; };   // lanes
+    int block = 256;
+    if (fullest(128) * 5 <= fullest(block) * 4) block = 128;
+    if (fullest(64) * 23 <= fullest(block) * 20) block = 64;
+    return block;
+}
+
 // Shared launch logic: choose the kernel for (prec, sr), size the grid from
 // occupancy (persistent: enough lanes to fill the GPU, no more than the work).
 template <class ModelF>
@@ -108,14 +130,12 @@ cudaError_t launch_family(const RunArgs &a, int prec, int sr, LaunchConfig cfg, 
     if (e != cudaSuccess) return e;
     int block = cfg.block;
     if (block == 0) {
-        // 256 threads (eight warps per block pack better under tail compaction)
-        // unless they keep fewer than 85% of the warps 128-thread blocks would
         int p256 = 0, p128 = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p256, k, 256, 0);
         if (e != cudaSuccess) return e;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p128, k, 128, 0);
         if (e != cudaSuccess) return e;
-        block = (p256 * 8 * 100 >= p128 * 4 * 85) ? 256 : 128;
+        block = default_block(a.n_work, sms, p256, p128);
     }
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, 0);
     if (e != cudaSuccess) return e;
