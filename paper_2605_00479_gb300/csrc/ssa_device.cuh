@@ -52,6 +52,10 @@ constexpr int kMaxK = 1024;
 #define SSA_MIN_BLOCKS 1
 #endif
 
+#ifndef SSA_KERNEL_BUDGETS
+#define SSA_KERNEL_BUDGETS 1   // 0: every kernel at SSA_MIN_BLOCKS (for comparisons)
+#endif
+
 // Per kernel: a register budget, as 256-thread blocks per SM, where it was
 // measured to pay.  The one-species birth-death structure's round-to-nearest
 // kernels (not fp64) fit 64 registers: four blocks, 9.6 ms for 10^6
@@ -60,13 +64,19 @@ constexpr int kMaxK = 1024;
 // than the compiler's choice (three / four / five blocks: Schloegl mixed bf16
 // +4 / +6 / +4%, uniform f16 SR +6 / +21 / +27%, telegraph +6 / +5 / +6%,
 // repressilator +4 / +11 / +23%).
-#ifndef SSA_KERNEL_BUDGETS
-#define SSA_KERNEL_BUDGETS 1   // 0: every kernel at SSA_MIN_BLOCKS (for comparisons)
-#endif
 
+//
+// General networks: three blocks (80 registers) except in fp64 and uniform SR.
+// 10^5 trajectories of a six-reaction network, fp32: 36.6 ms without a budget,
+// 23.8 / 24.6 ms at three / four blocks; repressilator with h = 3, mixed f16,
+// 51.9, 40.9 / 41.5; uniform f16 SR (10^4) 34.7, 38.9 / 41.4; fp64 7.5, 7.9 / 7.9.
 template <class Model, int PREC, int SR>
 struct KernelMinBlocks {
-        static constexpr int value = (SSA_KERNEL_BUDGETS && Model::N == 1 && SR == 0 && PREC != 0) ? 4 : SSA_MIN_BLOCKS;
+    static constexpr bool kGeneral = Model::N == kMaxN && Model::M == kMaxM;
+    static constexpr bool kUniformSR = SR == 1 && (PREC == 4 || PREC == 5);
+    static constexpr int value = !SSA_KERNEL_BUDGETS ? SSA_MIN_BLOCKS
+                                 : kGeneral          ? (PREC != 0 && !kUniformSR ? 3 : SSA_MIN_BLOCKS)
+                                 : (Model::N == 1 && SR == 0 && PREC != 0) ? 4 : SSA_MIN_BLOCKS;
 };
 
 enum Precision { FP64 = 0, FP32 = 1, MIXED_F16 = 2, MIXED_BF16 = 3, UNIFORM_F16 = 4, UNIFORM_BF16 = 5 };
@@ -529,6 +539,44 @@ __device__ __forceinline__ void store_state(const RunArgs &a, int k, int64_t ite
     });
 }
 
+// The general model's state lies in local memory: one out-of-line copy with a
+// loop keeps its callers' registers (ssa_step_general: five inlined copies of
+// the unrolled form cost the whole kernel 30 registers).
+template <class Model>
+__device__ __noinline__ uint32_t store_state_loop(const RunArgs &a, int k, int64_t item, const int *x, uint32_t status)
+{
+    int row = 0;
+#pragma unroll 1
+    for (int i = 0; i < a.N; ++i) {
+        if (!((a.out_mask >> i) & 1u)) continue;
+        const int64_t idx = ((int64_t)k * a.out_N + row) * a.n_traj + item;
+        int v = x[i];
+        if (a.state_bytes == 2) {
+            if (v > 32767) { v = 32767; status |= ST_STATE_RANGE; }
+            if (v < -32768) { v = -32768; status |= ST_STATE_RANGE; }
+            static_cast<int16_t *>(a.out)[idx] = (int16_t)v;
+        } else {
+            static_cast<int32_t *>(a.out)[idx] = v;
+        }
+        row += 1;
+    }
+    return status;
+}
+
+template <int PREC>
+__device__ __noinline__ void finish_general(const RunArgs &a, Lane<GeneralModel, PREC> &L)
+{
+#pragma unroll 1
+    while (L.k < a.K) {
+        L.status = store_state_loop<GeneralModel>(a, L.k, L.item, L.x, L.status);
+        L.k += 1;
+    }
+    a.status[L.item] = L.status;
+    if (a.n_events) a.n_events[L.item] = L.n;
+    if (a.t_final) a.t_final[L.item] = (double)L.t;
+    L.active = false;
+}
+
 template <class Model, int PREC>
 __device__ void finish(const RunArgs &a, Lane<Model, PREC> &L)
 {
@@ -543,10 +591,43 @@ __device__ void finish(const RunArgs &a, Lane<Model, PREC> &L)
 }
 
 // ------------------------------------------------------------ lane refill
+// init_lane for the general model (state in local memory): one copy, loops.
+template <int PREC>
+__device__ __noinline__ void init_general(const RunArgs &a, Lane<GeneralModel, PREC> &L, int64_t item, double s_first)
+{
+    using P = typename ModeTraits<PREC>::P;
+    L.item = item;
+    L.traj = a.traj_offset + (uint32_t)item;
+    const int64_t set = a.n_sets > 1 ? item / a.traj_per_set : 0;
+#pragma unroll 1
+    for (int i = 0; i < a.N; ++i) L.x[i] = a.x0_tab ? a.x0_tab[set * a.N + i] : a.x0[i];
+#pragma unroll 1
+    for (int j = 0; j < a.M; ++j) {
+        L.c[j] = to_prop<PREC>(a.n_sets > 1 ? a.cprime_tab[set * a.M + j] : a.cprime[j]);
+        L.h0[j] = P(0);
+        L.h1[j] = P(0);
+        if (a.law[j] == 1) {
+            const bool tab = a.n_sets > 1 && a.hill_tab;
+            L.h0[j] = to_prop<PREC>(tab ? a.hill_tab[(set * a.M + j) * 2 + 0] : a.hill_a0[j]);
+            L.h1[j] = to_prop<PREC>(tab ? a.hill_tab[(set * a.M + j) * 2 + 1] : a.hill_a[j]);
+        }
+    }
+    L.t = P(0);
+    L.n = 0;
+    L.k = 0;
+    L.status = 0;
+    L.s_next = (P)s_first;
+    L.active = true;
+}
+
 template <class Model, int PREC>
 __device__ void init_lane(const RunArgs &a, Lane<Model, PREC> &L, int64_t item, const typename ModeTraits<PREC>::P *smp)
 {
     using P = typename ModeTraits<PREC>::P;
+    if constexpr (std::is_same<Model, GeneralModel>::value) {
+        init_general<PREC>(a, L, item, a.K > 0 ? (double)smp[0] : (double)__int_as_float(0x7F800000));
+        return;
+    }
     L.item = item;
     L.traj = a.traj_offset + (uint32_t)item;
     const int set = a.n_sets > 1 ? (int)(item / a.traj_per_set) : 0;
@@ -898,7 +979,7 @@ __device__ __noinline__ void ssa_step_general(const RunArgs &a, Lane<GeneralMode
             return;
         }
         L.status |= ST_MAX_EVENTS;
-        finish<GeneralModel, PREC>(a, L);
+        finish_general<PREC>(a, L);
         return;
     }
     Rounder<PREC, SR> R;
@@ -926,9 +1007,9 @@ __device__ __noinline__ void ssa_step_general(const RunArgs &a, Lane<GeneralMode
         }
     }
     const P a0 = S[a.M - 1];
-    if (is_nan<PREC>(a0)) { L.status |= ST_NAN; finish<GeneralModel, PREC>(a, L); return; }
-    if (a0 == kInf) { L.status |= ST_OVERFLOW; finish<GeneralModel, PREC>(a, L); return; }
-    if (a0 == P(0)) { finish<GeneralModel, PREC>(a, L); return; }
+    if (is_nan<PREC>(a0)) { L.status |= ST_NAN; finish_general<PREC>(a, L); return; }
+    if (a0 == kInf) { L.status |= ST_OVERFLOW; finish_general<PREC>(a, L); return; }
+    if (a0 == P(0)) { finish_general<PREC>(a, L); return; }
 
     P tau, target, t_new;
     if constexpr (Tr::kF64) {
@@ -956,11 +1037,11 @@ __device__ __noinline__ void ssa_step_general(const RunArgs &a, Lane<GeneralMode
         }
     }
     while (L.s_next < t_new) {
-        store_state<GeneralModel>(a, L.k, L.item, L.x, L.status);
+        L.status = store_state_loop<GeneralModel>(a, L.k, L.item, L.x, L.status);
         L.k += 1;
         L.s_next = L.k < a.K ? smp[L.k] : kInf;
     }
-    if (t_new > t_end) { finish<GeneralModel, PREC>(a, L); return; }
+    if (t_new > t_end) { finish_general<PREC>(a, L); return; }
 
     int mu = -1;
 #pragma unroll 1
@@ -981,7 +1062,7 @@ __device__ __noinline__ void ssa_step_general(const RunArgs &a, Lane<GeneralMode
     L.n += 1;
     if (negative) {
         L.status |= ST_STATE_RANGE;
-        finish<GeneralModel, PREC>(a, L);
+        finish_general<PREC>(a, L);
     }
 }
 
@@ -1246,6 +1327,7 @@ __device__ __forceinline__ void run_queue(const RunArgs &a, const typename ModeT
 }  // namespace ssa
 
 #include "ssa_fast.cuh"
+#include "ssa_general.cuh"
 
 namespace ssa {
 
@@ -1257,6 +1339,34 @@ __device__ __forceinline__ void run_any(const RunArgs &a, const typename ModeTra
 {
     if constexpr (std::is_same<Model, GeneralModel>::value) run_queue<Model, PREC, SR>(a, smp, t_end, pool);
     else run_queue_fast<Model, PREC, SR>(a, smp, t_end, ln2, pool);
+}
+
+// Single-model launches: the structure lists of a general network.  A launch
+// over several parameter sets of one keeps ssa_step_general (its constants
+// differ from lane to lane).
+template <class Model, int PREC>
+struct KernelTables {
+    using type = int;
+};
+template <int PREC>
+struct KernelTables<GeneralModel, PREC> {
+    using type = GeneralTables<PREC>;
+};
+
+template <class Model, int PREC, int SR>
+__device__ __forceinline__ void run_single(const RunArgs &a, const typename ModeTraits<PREC>::P *smp,
+                                           typename ModeTraits<PREC>::P t_end, const double2 *ln2,
+                                           const typename KernelTables<Model, PREC>::type *tables,
+                                           TailPool<Model, PREC> *pool)
+{
+    extern __shared__ __align__(16) unsigned char columns[];   // general_columns bytes
+    if constexpr (std::is_same<Model, GeneralModel>::value) {
+        if (a.n_sets == 1) {
+            run_queue_general<PREC, SR>(a, smp, t_end, ln2, *tables, columns, pool);
+            return;
+        }
+    }
+    run_any<Model, PREC, SR>(a, smp, t_end, ln2, pool);
 }
 
 template <int PREC>
@@ -1281,8 +1391,10 @@ __global__ void __launch_bounds__(256, (KernelMinBlocks<Model, PREC, SR>::value)
     const bool pooled = a.tail_stats != nullptr;
     if (pooled) pool_init(&pool);
     load_samples<PREC>(a.samples, a.K, smp, ln2);   // ends with __syncthreads
+    __shared__ typename KernelTables<Model, PREC>::type tables;
+    if constexpr (std::is_same<Model, GeneralModel>::value) build_general_tables<PREC>(a, &tables);
     for (int pass = 0;; ++pass) {
-        run_any<Model, PREC, SR>(a, smp, to_time<PREC>(a.t_end), ln2, pooled ? &pool : nullptr);
+        run_single<Model, PREC, SR>(a, smp, to_time<PREC>(a.t_end), ln2, &tables, pooled ? &pool : nullptr);
         if (!pooled || pass > 0) break;
         // every warp has left the loop: records stranded by a lock wait that
         // gave up are resumed by warp 0 (the pool no longer changes)

@@ -128,16 +128,24 @@ cudaError_t launch_family(const RunArgs &a, int prec, int sr, LaunchConfig cfg, 
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    // dynamic shared memory: the columns of a general network's lanes (at most 41 KB)
+    auto columns = [&](int b) -> size_t {
+        return std::is_same<ModelF, GeneralModel>::value && a.n_sets == 1 ? general_columns(a.N, a.M, prec, b) : 0;
+    };
+    if (columns(256) > 0) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)columns(256));
+        if (e != cudaSuccess) return e;
+    }
     int block = cfg.block;
     if (block == 0) {
         int p256 = 0, p128 = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p256, k, 256, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p256, k, 256, columns(256));
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p128, k, 128, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p128, k, 128, columns(128));
         if (e != cudaSuccess) return e;
         block = default_block(a.n_work, sms, p256, p128);
     }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, columns(block));
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     if (cfg.blocks_per_sm > 0 && cfg.blocks_per_sm < per_sm) per_sm = cfg.blocks_per_sm;
@@ -146,7 +154,7 @@ cudaError_t launch_family(const RunArgs &a, int prec, int sr, LaunchConfig cfg, 
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
     *grid_out = (int)grid;
-    k<<<(unsigned)grid, (unsigned)block, 0, stream>>>(a);
+    k<<<(unsigned)grid, (unsigned)block, columns(block), stream>>>(a);
     return cudaGetLastError();
 }
 
