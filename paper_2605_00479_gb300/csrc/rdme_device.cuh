@@ -134,6 +134,7 @@ template <int PREC>
 struct RLane {
     using P = typename ModeTraits<PREC>::P;
     P t, s_next;
+    P a0, lim;             // compiled structures: the root, the earlier of the next sample and t_end
     int64_t n, item;
     uint32_t traj, status;
     int k;
@@ -202,10 +203,10 @@ struct ChannelSum {
     }
 };
 
-// Voxel v at epoch e: returns its total; with sel, also the channel selected
-// by residual target r.
-template <class Model, int PREC, int SR>
-__device__ __forceinline__ typename ModeTraits<PREC>::P rdme_voxel(const RdmeArgs &A, const RdmeView<PREC> &W, int v,
+// General model.  Voxel v at epoch e: returns its total; with sel, also the
+// channel selected by residual target r.
+template <int PREC, int SR>
+__device__ __forceinline__ typename ModeTraits<PREC>::P rdme_voxel_general(const RdmeArgs &A, const RdmeView<PREC> &W, int v,
                                                                    uint32_t e, uint32_t traj,
                                                                    typename ModeTraits<PREC>::P r, int *sel)
 {
@@ -231,125 +232,176 @@ __device__ __forceinline__ typename ModeTraits<PREC>::P rdme_voxel(const RdmeArg
     cs.mu = -1;
     cs.last_pos = -1;
 
-    if constexpr (RdmeSpecies<Model>::kStatic) {
-        constexpr int M = Model::M, N = Model::N;
-        P prop[M];
-        unroll<M>([&](auto J) {
-            constexpr int j = decltype(J)::value;
-            int op = Model::template chain_start<j>(a);
-            if (Model::template law<j>(a) == 1) {
-                const int reg = Model::template hill_reg<j>(a);
-                int xr = 0;
-                unroll<N>([&](auto I) {
-                    constexpr int i = decltype(I)::value;
-                    if (i == reg) xr = rdme_get<Model, i>(W, v);
-                });
-                const P Pv = R.rnd((P)xr, op++);
-                P q = Pv;
-                const int h = Model::template hill_h<j>(a);
-                for (int m = 1; m < h; ++m) q = R.rnd(q * Pv, op++);
-                const P d = R.rnd(P(1) + q, op++);
-                const P f = R.rnd(W.h1P[j] / d, op++);
-                prop[j] = R.rnd(W.h0P[j] + f, op++);
-            } else {
-                P av = W.cP[j];
-                bool zero = false;
-                unroll<N>([&](auto I) {
-                    constexpr int i = decltype(I)::value;
-                    const int rr = Model::template order<j, i>(a);
-                    if (rr > 0 && !Model::template folded<j, i>(a)) {
-                        const int xi = rdme_get<Model, i>(W, v);
-                        zero = zero || (xi < rr);
-                        for (int m = 0; m < rr; ++m) {
-                            const P f = R.rnd((P)(xi - m), op++);
-                            av = R.rnd(av * f, op++);
-                        }
-                    }
-                });
-                prop[j] = zero ? P(0) : av;
-            }
-        });
-        P hv[N];
-        int op = Model::total_chain_ops(a);
-        unroll<N>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            hv[i] = P(0);
-            if (nnb > 0 && ((W.dmask >> i) & 1u)) {
-                const int xi = rdme_get<Model, i>(W, v);
-                if (xi < 1) {
-                    op += 2;
-                } else {
-                    const P f = R.rnd((P)xi, op++);
-                    hv[i] = R.rnd(W.DP[i] * f, op++);
-                }
-            }
-        });
-        cs.op0 = op;
-        unroll<M>([&](auto J) { cs.add(prop[decltype(J)::value]); });
-        if (nnb > 0) {
-            unroll<N>([&](auto I) {
-                constexpr int i = decltype(I)::value;
-                if ((W.dmask >> i) & 1u)
-                    for (int d = 0; d < nnb; ++d) cs.add(hv[i]);
-            });
-        }
-    } else {
-        const int N = a.N, M = a.M;
-        P prop[kMaxM];
+    const int N = a.N, M = a.M;
+    P prop[kMaxM];
 #pragma unroll 1
-        for (int j = 0; j < M; ++j) {
-            int op = a.chain_start[j];
-            if (a.law[j] == 1) {
-                const P Pv = R.rnd((P)W.at(v, a.hill_reg[j]), op++);
-                P q = Pv;
-                for (int m = 1; m < a.hill_h[j]; ++m) q = R.rnd(q * Pv, op++);
-                const P d = R.rnd(P(1) + q, op++);
-                const P f = R.rnd(W.h1P[j] / d, op++);
-                prop[j] = R.rnd(W.h0P[j] + f, op++);
-            } else {
-                P av = W.cP[j];
-                bool zero = false;
-#pragma unroll 1
-                for (int i = 0; i < N; ++i) {
-                    const int rr = a.order[j][i];
-                    if (rr == 0 || a.folded[j][i]) continue;
-                    const int xi = W.at(v, i);
-                    zero = zero || (xi < rr);
-                    for (int m = 0; m < rr; ++m) {
-                        const P f = R.rnd((P)(xi - m), op++);
-                        av = R.rnd(av * f, op++);
-                    }
-                }
-                prop[j] = zero ? P(0) : av;
-            }
-        }
-        P hv[kMaxN];
-        int op = a.sr_ops;
-#pragma unroll 1
-        for (int i = 0; i < N; ++i) {
-            hv[i] = P(0);
-            if (nnb == 0 || !((W.dmask >> i) & 1u)) continue;
-            const int xi = W.at(v, i);
-            if (xi < 1) {
-                op += 2;
-            } else {
-                const P f = R.rnd((P)xi, op++);
-                hv[i] = R.rnd(W.DP[i] * f, op++);
-            }
-        }
-        cs.op0 = op;
-#pragma unroll 1
-        for (int j = 0; j < M; ++j) cs.add(prop[j]);
-        if (nnb > 0) {
+    for (int j = 0; j < M; ++j) {
+        int op = a.chain_start[j];
+        if (a.law[j] == 1) {
+            const P Pv = R.rnd((P)W.at(v, a.hill_reg[j]), op++);
+            P q = Pv;
+            for (int m = 1; m < a.hill_h[j]; ++m) q = R.rnd(q * Pv, op++);
+            const P d = R.rnd(P(1) + q, op++);
+            const P f = R.rnd(W.h1P[j] / d, op++);
+            prop[j] = R.rnd(W.h0P[j] + f, op++);
+        } else {
+            P av = W.cP[j];
+            bool zero = false;
 #pragma unroll 1
             for (int i = 0; i < N; ++i) {
-                if (!((W.dmask >> i) & 1u)) continue;
-                for (int d = 0; d < nnb; ++d) cs.add(hv[i]);
+                const int rr = a.order[j][i];
+                if (rr == 0 || a.folded[j][i]) continue;
+                const int xi = W.at(v, i);
+                zero = zero || (xi < rr);
+                for (int m = 0; m < rr; ++m) {
+                    const P f = R.rnd((P)(xi - m), op++);
+                    av = R.rnd(av * f, op++);
+                }
             }
+            prop[j] = zero ? P(0) : av;
+        }
+    }
+    P hv[kMaxN];
+    int op = a.sr_ops;
+#pragma unroll 1
+    for (int i = 0; i < N; ++i) {
+        hv[i] = P(0);
+        if (nnb == 0 || !((W.dmask >> i) & 1u)) continue;
+        const int xi = W.at(v, i);
+        if (xi < 1) {
+            op += 2;
+        } else {
+            const P f = R.rnd((P)xi, op++);
+            hv[i] = R.rnd(W.DP[i] * f, op++);
+        }
+    }
+    cs.op0 = op;
+#pragma unroll 1
+    for (int j = 0; j < M; ++j) cs.add(prop[j]);
+    if (nnb > 0) {
+#pragma unroll 1
+        for (int i = 0; i < N; ++i) {
+            if (!((W.dmask >> i) & 1u)) continue;
+            for (int d = 0; d < nnb; ++d) cs.add(hv[i]);
         }
     }
     if (sel) *sel = cs.mu >= 0 ? cs.mu : cs.last_pos;
     return cs.S;
+}
+
+// ------------------------------------------------ voxels of compiled structures
+// Counts of one voxel, read once (held species from the block's table).
+template <class Model>
+struct VoxelCounts {
+    int x[Model::N];
+    template <int I> __device__ __forceinline__ float f(int m) const { return (float)(x[I] - m); }
+    template <int I> __device__ __forceinline__ double d(int m) const
+    {
+        const int v = x[I] - m;
+        return v < (1 << 24) ? count_f64((float)v) : (double)v;
+    }
+    template <int I> __device__ __forceinline__ bool below(int r) const { return x[I] < r; }
+};
+
+// What a lane needs of the network beside its own state: the propensity
+// constants in registers (one parameter set: the same for every lattice).
+template <class Model, int PREC, int SR>
+struct VoxelModel {
+    FastLane<Model, PREC, SR> L;
+    bool odd;
+};
+
+template <int PREC, int SR>
+struct VoxelModel<GeneralModel, PREC, SR> {
+};
+
+// Voxel v at epoch e: its total; with SEL also the channel *sel whose partial
+// sum first exceeds r (the sums never decrease, so it is the number of sums
+// at or below r; none: the last channel with a positive value, -1 if none).
+template <bool SEL, class Model, int PREC, int SR>
+__device__ __forceinline__ typename ModeTraits<PREC>::P rdme_voxel_fast(const RdmeArgs &A, const RdmeView<PREC> &W,
+                                                                        const VoxelModel<Model, PREC, SR> &C, int v, uint32_t e,
+                                                                        uint32_t traj, typename ModeTraits<PREC>::P r, int *sel)
+{
+    using Tr = ModeTraits<PREC>;
+    using P = typename Tr::P;
+    constexpr int M = Model::M, N = Model::N, kFmt = Tr::kFmt;
+    const RunArgs &a = A.a;
+    TagBits bits;
+    if constexpr (Tr::k16 && SR) {
+        bits.e = e;
+        bits.traj = traj;
+        bits.tag = 0x80000000u | (uint32_t)v;
+        bits.k0 = a.key0;
+        bits.k1 = a.key1;
+        bits.cur = -1;
+    }
+    auto rnd = [&](P x, int op) -> P {
+        if constexpr (!Tr::k16) return x;
+        else if constexpr (SR != 0) return sr16<kFmt>(x, bits.word(op), (op & 1) != 0);
+        else return rn16<kFmt>(x);
+    };
+    VoxelCounts<Model> X;
+    unroll<N>([&](auto I) { X.x[decltype(I)::value] = rdme_get<Model, decltype(I)::value>(W, v); });
+    P prop[M];
+    uint16_t p16[M];
+    fast_propensities<true>(C.L, X, bits, prop, p16, C.odd);
+    const int nnb = __popc((unsigned)W.nbmask[v]);
+    P hv[N];
+    int op = ChainPlan<Model>::first_slot(M);
+    unroll<N>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        hv[i] = P(0);
+        if (((W.dmask >> i) & 1u) && nnb > 0) {
+            P f;
+            if constexpr (Tr::kF64) f = X.x[i] < (1 << 24) ? count_f64((float)X.x[i]) : (double)X.x[i];
+            else f = rnd((P)X.x[i], op);
+            f = rnd(W.DP[i] * f, op + 1);
+            hv[i] = X.x[i] < 1 ? P(0) : f;
+            op += 2;
+        }
+    });
+    P S = prop[0];
+    int at_or_below = 0, c = 0;
+    auto passed = [&]() {
+        if constexpr (SEL) at_or_below += later(S, r) ? 0 : 1;
+    };
+    passed();
+    unroll<M - 1>([&](auto J) {
+        constexpr int j = decltype(J)::value + 1;
+        if constexpr (Tr::kUniform) S = rnd(S + prop[j], op + j - 1);
+        else S = S + prop[j];
+        passed();
+    });
+    c = M;
+    unroll<N>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        if ((W.dmask >> i) & 1u) {
+            for (int d = 0; d < nnb; ++d) {
+                if constexpr (Tr::kUniform) S = rnd(S + hv[i], op + c - 1);
+                else S = S + hv[i];
+                c += 1;
+                passed();
+            }
+        }
+    });
+    if constexpr (SEL) {
+        int mu = at_or_below;
+        if (mu == c) {
+            mu = -1;
+            unroll<M>([&](auto J) { if (prop[decltype(J)::value] > P(0)) mu = decltype(J)::value; });
+            int q = M;
+            unroll<N>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                if ((W.dmask >> i) & 1u) {
+                    q += nnb;
+                    if (hv[i] > P(0) && nnb > 0) mu = q - 1;
+                }
+            });
+        }
+        *sel = mu;
+    }
+    return S;
 }
 
 // Tree node q at epoch e from its children's values (left + right).
@@ -425,7 +477,8 @@ __device__ void rdme_finish(const RdmeArgs &A, const RdmeView<PREC> &W, RLane<PR
 }
 
 template <class Model, int PREC, int SR>
-__device__ void rdme_init(const RdmeArgs &A, const RdmeView<PREC> &W, RLane<PREC> &L, int64_t item)
+__device__ void rdme_init(const RdmeArgs &A, const RdmeView<PREC> &W, const VoxelModel<Model, PREC, SR> &C, RLane<PREC> &L,
+                          int64_t item)
 {
     using P = typename ModeTraits<PREC>::P;
     const int N = A.a.N;
@@ -446,11 +499,18 @@ __device__ void rdme_init(const RdmeArgs &A, const RdmeView<PREC> &W, RLane<PREC
     }
 #pragma unroll 1
     for (int v = 0; v < A.T; ++v) {
-        W.Node(A.T + v) = v < A.S ? rdme_voxel<Model, PREC, SR>(A, W, v, 0u, L.traj, P(0), nullptr) : P(0);
+        P total = P(0);
+        if (v < A.S) {
+            if constexpr (RdmeSpecies<Model>::kStatic)
+                total = rdme_voxel_fast<false>(A, W, C, v, 0u, L.traj, P(0), nullptr);
+            else total = rdme_voxel_general<PREC, SR>(A, W, v, 0u, L.traj, P(0), nullptr);
+        }
+        W.Node(A.T + v) = total;
         if (W.epoch && v < A.S) W.epoch[v * W.bd] = 0u;
     }
 #pragma unroll 1
     for (int q = A.T - 1; q >= 1; --q) W.Node(q) = rdme_node<PREC, SR>(A, W, q, 0u, L.traj);
+    L.a0 = W.Node(1);
     L.t = P(0);
     L.n = 0;
     L.k = 0;
@@ -539,7 +599,7 @@ __device__ __forceinline__ int rdme_apply(const RdmeArgs &A, const RdmeView<PREC
     return w;
 }
 
-// One event of an active lane (contract above).
+// One event of an active lane (contract above), general model.
 template <class Model, int PREC, int SR>
 __device__ __forceinline__ void rdme_event(const RdmeArgs &A, const RdmeView<PREC> &W, RLane<PREC> &L,
                                            typename ModeTraits<PREC>::P t_end)
@@ -648,7 +708,7 @@ __device__ __forceinline__ void rdme_event(const RdmeArgs &A, const RdmeView<PRE
     const int v = q - T;
     const uint32_t ev = W.epoch ? W.epoch[v * W.bd] : 0u;
     int c = -1;
-    rdme_voxel<Model, PREC, SR>(A, W, v, ev, L.traj, r, &c);
+    rdme_voxel_general<PREC, SR>(A, W, v, ev, L.traj, r, &c);
     if (c < 0) {            // unreachable (the descent enters only positive totals); kept as a guard
         L.status |= ST_NAN;
         rdme_finish<Model, PREC>(A, W, L);
@@ -681,12 +741,12 @@ __device__ __forceinline__ void rdme_event(const RdmeArgs &A, const RdmeView<PRE
         }
     }
     const uint32_t e = (uint32_t)L.n;
-    P va = rdme_voxel<Model, PREC, SR>(A, W, v, e, L.traj, P(0), nullptr);
+    P va = rdme_voxel_general<PREC, SR>(A, W, v, e, L.traj, P(0), nullptr);
     W.Node(la) = va;
     if (W.epoch) W.epoch[v * W.bd] = e;
     P vb = P(0);
     if (w >= 0) {
-        vb = rdme_voxel<Model, PREC, SR>(A, W, w, e, L.traj, P(0), nullptr);
+        vb = rdme_voxel_general<PREC, SR>(A, W, w, e, L.traj, P(0), nullptr);
         W.Node(lb) = vb;
         if (W.epoch) W.epoch[w * W.bd] = e;
     }
@@ -715,6 +775,193 @@ __device__ __forceinline__ void rdme_event(const RdmeArgs &A, const RdmeView<PRE
     }
 }
 
+// One event, compiled structures.  What bounds it is instruction count (the
+// columns are conflict-free shared memory): the arithmetic is that of
+// ssa_fast.cuh, a changed leaf climbs the tree with one addition a level (a
+// node is the sum of two, in either order), and a hop's destination climbs
+// first, so both paths' common part ends with the final values.  Measured
+// (GB300, 32-voxel Schloegl chain, mixed f16, 65536 lattices): 64.1 -> 53.8 ms;
+// mixed f16 SR 59.7 -> 46.6 ms (to t = 0.1).  E: -log u1; w1: the second word.
+template <class Model, int PREC>
+__device__ __forceinline__ int rdme_hop_target(const RdmeArgs &A, unsigned nb, int v, int idx)
+{
+    for (int q = 0; q < idx; ++q) nb &= nb - 1u;
+    return rdme_neighbour(A, v, __ffs((int)nb) - 1);
+}
+
+template <int PREC, int SR>
+__device__ __forceinline__ typename ModeTraits<PREC>::P rdme_climb(const RdmeArgs &A, const RdmeView<PREC> &W, int leaf,
+                                                                   typename ModeTraits<PREC>::P val, uint32_t e, uint32_t traj)
+{
+    using P = typename ModeTraits<PREC>::P;
+    int q = leaf;
+    W.Node(q) = val;
+    P sib = A.depth > 0 ? W.Node(q ^ 1) : P(0);
+#pragma unroll 1
+    for (int l = 0; l < A.depth; ++l) {
+        const int up = q >> 1;
+        const P s = sib;
+        if (l + 1 < A.depth) sib = W.Node(up ^ 1);   // the next level's, ahead of this level's store
+        val = rdme_sum<PREC, SR>(A, val, s, up, e, traj);
+        W.Node(up) = val;
+        q = up;
+    }
+    return val;
+}
+
+template <class Model, int PREC, int SR>
+__device__ __forceinline__ void rdme_event_fast(const RdmeArgs &A, const RdmeView<PREC> &W,
+                                                const VoxelModel<Model, PREC, SR> &C, RLane<PREC> &L,
+                                                typename ModeTraits<PREC>::P E, uint32_t w1, typename ModeTraits<PREC>::P t_end)
+{
+    using Tr = ModeTraits<PREC>;
+    using P = typename Tr::P;
+    constexpr int M = Model::M, N = Model::N;
+    const RunArgs &a = A.a;
+    const P a0 = L.a0;
+    Rounder<PREC, SR> R;   // event-level operations (uniform modes)
+    if constexpr (Tr::kUniform && SR) {
+        R.bits.base = (uint64_t)L.n * (uint64_t)((5 + A.depth + 7) >> 3);
+        R.bits.traj = L.traj;
+        R.bits.k0 = a.key0;
+        R.bits.k1 = a.key1;
+        R.bits.cur = -1;
+    }
+    uint32_t ab;
+    constexpr uint32_t kLow = Tr::kF64 ? 0x07B00000u : 0x12800000u;     // as in fast_step
+    constexpr uint32_t kSpan = Tr::kF64 ? 0x70800000u : 0x5A000000u;
+    if constexpr (Tr::kF64) ab = (uint32_t)__double2hiint(a0);
+    else ab = __float_as_uint(a0);
+    const bool wild = ab - kLow > kSpan;
+    P target, t_new;
+    if constexpr (Tr::kF64) {
+        target = u32_scaled(w1) * a0;
+        t_new = L.t + E / a0;
+    } else {
+        const float u2 = (float)(w1 >> 8) * 0x1p-24f;
+        if constexpr (Tr::kUniform) {
+            const float Er = R.rnd(E, 0);
+            const float U2 = R.rnd(u2, 1);
+            const float tau = R.rnd(wild ? Er / a0 : div_short(Er, a0), 2);
+            target = R.rnd(U2 * a0, 3);
+            t_new = R.rnd(L.t + tau, 4);
+        } else {
+            target = u2 * a0;
+            t_new = L.t + (wild ? E / a0 : div_rn(E, a0));
+        }
+    }
+    const bool due = later(t_new, L.lim);
+    if (wild || due || L.n >= a.max_events) {
+        const P kInf = P(__int_as_float(0x7F800000));
+        bool ends = true;
+        if (L.n >= a.max_events) L.status |= ST_MAX_EVENTS;
+        else if (a0 != a0) L.status |= ST_NAN;
+        else if (a0 == kInf) L.status |= ST_OVERFLOW;
+        else if (a0 != P(0)) {
+            while (L.k < a.K && later(t_new, W.smp[L.k])) {
+                rdme_store<Model, PREC>(A, W, L.k, L.item, L.status);
+                L.k += 1;
+            }
+            const P s_next = L.k < a.K ? W.smp[L.k] : t_end;
+            L.lim = later(s_next, t_end) ? t_end : s_next;
+            ends = later(t_new, t_end);
+        }
+        if (ends) rdme_finish<Model, PREC>(A, W, L);
+    }
+    if (!L.active) return;
+
+    // voxel by descent of the sum tree, two levels per round of reads
+    const int T = A.T;
+    int q = 1, level = 0;
+    P r = target;
+    auto down = [&](P lf, P rt) {
+        const bool right = !later(lf, r) && later(rt, P(0));
+        if constexpr (Tr::kUniform && SR != 0) {
+            if (right) r = R.rnd(r - lf, 5 + level);
+        } else {
+            P d = r - lf;
+            if constexpr (Tr::kUniform) d = rn16<Tr::kFmt>(d);
+            r = right ? d : r;
+        }
+        q = 2 * q + (right ? 1 : 0);
+        level += 1;
+        return right;
+    };
+#pragma unroll 1
+    while (q < T) {
+        const P lf = W.Node(2 * q), rt = W.Node(2 * q + 1);
+        if (2 * q < T) {   // children internal: their children are read along
+            const P g0 = W.Node(4 * q), g1 = W.Node(4 * q + 1), g2 = W.Node(4 * q + 2), g3 = W.Node(4 * q + 3);
+            const bool right = down(lf, rt);
+            down(right ? g2 : g0, right ? g3 : g1);
+        } else {
+            down(lf, rt);
+        }
+    }
+    const int v = q - T;
+    const uint32_t ev = W.epoch ? W.epoch[v * W.bd] : 0u;
+    int c = -1;
+    rdme_voxel_fast<true>(A, W, C, v, ev, L.traj, r, &c);
+    if (c < 0) {            // unreachable (the descent enters only positive totals); kept as a guard
+        L.status |= ST_NAN;
+        rdme_finish<Model, PREC>(A, W, L);
+        return;
+    }
+    // apply channel c: a reaction's changes by selects, or a hop
+    const unsigned nb = W.nbmask[v];
+    const int nnb = __popc(nb);
+    int w = -1;
+    bool negative = false;
+    if (c < M) {
+        unroll<N>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            constexpr int s = RdmeSpecies<Model>::slot(i);
+            if constexpr (s >= 0 && ChainPlan<Model>::moves(i)) {
+                int d = 0;
+                unroll<M>([&](auto J) {
+                    constexpr int j = decltype(J)::value;
+                    const int nu = Model::template nu<j, i>(a);
+                    if (nu != 0) d = c == j ? nu : d;
+                });
+                int &xr = W.at(v, s);
+                xr += d;
+                negative = negative || xr < 0;
+            }
+        });
+    } else {
+        int idx = c - M;
+        unroll<N>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            constexpr int s = RdmeSpecies<Model>::slot(i);
+            if constexpr (s >= 0) {
+                if ((W.dmask >> i) & 1u) {
+                    if (idx >= 0 && idx < nnb) {
+                        w = rdme_hop_target<Model, PREC>(A, nb, v, idx);
+                        W.at(v, s) -= 1;
+                        W.at(w, s) += 1;
+                        negative = W.at(v, s) < 0;
+                    }
+                    idx -= nnb;
+                }
+            }
+        });
+    }
+    L.t = t_new;
+    L.n += 1;
+    if (negative) {
+        L.status |= ST_STATE_RANGE;
+        rdme_finish<Model, PREC>(A, W, L);
+        return;
+    }
+    const uint32_t e = (uint32_t)L.n;
+    if (w >= 0) {
+        if (W.epoch) W.epoch[w * W.bd] = e;
+        rdme_climb<PREC, SR>(A, W, T + w, rdme_voxel_fast<false>(A, W, C, w, e, L.traj, P(0), nullptr), e, L.traj);
+    }
+    if (W.epoch) W.epoch[v * W.bd] = e;
+    L.a0 = rdme_climb<PREC, SR>(A, W, T + v, rdme_voxel_fast<false>(A, W, C, v, e, L.traj, P(0), nullptr), e, L.traj);
+}
+
 // Persistent RDME kernel: lanes refill from the work queue; each loop
 // iteration runs up to kRdmeSlice events per lane.
 constexpr int kRdmeSlice = 8;
@@ -733,7 +980,7 @@ __global__ void __launch_bounds__(256) rdme_kernel(const __grid_constant__ RdmeA
     P *cons = reinterpret_cast<P *>(rdme_smem + lay.consts);
     int32_t *cst = reinterpret_cast<int32_t *>(rdme_smem + lay.cst);
     uint8_t *nbm = rdme_smem + lay.nbmask;
-    for (int k = tid; k < a.K; k += bd) smp[k] = to_time<PREC>(a.samples[k]);
+    for (int k = tid; k < a.K; k += bd) smp[k] = to_time<PREC>(a.samples[k]) + P(0);   // -0 becomes +0
     for (int j = tid; j < kMaxM; j += bd) {
         const bool on = j < a.M;
         cons[j] = on ? to_prop<PREC>(a.cprime[j]) : P(0);
@@ -778,6 +1025,11 @@ __global__ void __launch_bounds__(256) rdme_kernel(const __grid_constant__ RdmeA
     const unsigned lane = threadIdx.x & 31u;
     RLane<PREC> L;
     L.active = false;
+    VoxelModel<Model, PREC, SR> C;
+    if constexpr (RdmeSpecies<Model>::kStatic) {
+        fast_init(a, C.L, 0);      // the constants; a lattice has one parameter set
+        C.odd = C.L.odd;
+    }
     bool drained = false;
     for (;;) {
         const unsigned need = __ballot_sync(0xFFFFFFFFu, !L.active && !drained);
@@ -788,16 +1040,37 @@ __global__ void __launch_bounds__(256) rdme_kernel(const __grid_constant__ RdmeA
             base = __shfl_sync(0xFFFFFFFFu, base, leader);
             if (!L.active && !drained) {
                 const unsigned long long item = base + (unsigned long long)__popc(need & ((1u << lane) - 1u));
-                if (item < (unsigned long long)a.n_work) rdme_init<Model, PREC, SR>(A, W, L, (int64_t)item);
+                if (item < (unsigned long long)a.n_work) rdme_init<Model, PREC, SR>(A, W, C, L, (int64_t)item);
                 else drained = true;
             }
         }
         if (__ballot_sync(0xFFFFFFFFu, L.active) == 0u) break;
         // several events between refill checks (a lane that finishes idles
         // until the slice ends)
+        if constexpr (RdmeSpecies<Model>::kStatic) {
+            if (L.active) {
+                const P s_next = L.k < a.K ? smp[L.k] : t_end;
+                L.lim = later(s_next, t_end) ? t_end : s_next;
+            }
 #pragma unroll 1
-        for (int sl = 0; sl < kRdmeSlice; ++sl)
-            if (L.active) rdme_event<Model, PREC, SR>(A, W, L, t_end);
+            for (int sl = 0; sl < kRdmeSlice / 2; ++sl) {   // L.n is even for every active lane here
+                if (!L.active) continue;
+                const uint64_t blk = (uint64_t)L.n >> 1;
+                const uint4 u = philox4x32_10(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), L.traj, 0u), a.key0, a.key1);
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
+                    if (!L.active) break;
+                    P E;
+                    if constexpr (Tr::kF64) E = neg_log_u32(h ? u.z : u.x, nullptr);
+                    else E = neg_log_u24(((h ? u.z : u.x) >> 8) + 1u);
+                    rdme_event_fast<Model, PREC, SR>(A, W, C, L, E, h ? u.w : u.y, t_end);
+                }
+            }
+        } else {
+#pragma unroll 1
+            for (int sl = 0; sl < kRdmeSlice; ++sl)
+                if (L.active) rdme_event<Model, PREC, SR>(A, W, L, t_end);
+        }
     }
 }
 
