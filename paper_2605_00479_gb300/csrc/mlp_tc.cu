@@ -139,6 +139,62 @@ __device__ __forceinline__ void store_packed16(uint8_t *base, int64_t r, int c0,
     *reinterpret_cast<uint4 *>(base + packed_offset(r, c0 + 8, C)) = hi;
 }
 
+// 16 consecutive floats of one row.
+__device__ __forceinline__ void store16(float *p, const float (&v)[16], bool wide)
+{
+    if (wide) {
+#pragma unroll
+        for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4 *>(p + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) p[i] = v[i];
+    }
+}
+
+__device__ __forceinline__ void load16(const float *p, float (&v)[16], bool wide)
+{
+    if (wide) {
+#pragma unroll
+        for (int i = 0; i < 16; i += 4) {
+            const float4 q = *reinterpret_cast<const float4 *>(p + i);
+            v[i] = q.x; v[i + 1] = q.y; v[i + 2] = q.z; v[i + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = p[i];
+    }
+}
+
+// Sums of 16 columns over the warp's 32 rows: halving the columns a lane holds
+// with every exchange takes 16 shuffles instead of 80.  Lanes 2c and 2c + 1
+// return the sum of column c.
+__device__ __forceinline__ float column_sum16(const float (&v)[16], int lane)
+{
+    float a[8], b[4], c[2];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const bool up = (lane & 16) != 0;
+        const float keep = up ? v[i + 8] : v[i], give = up ? v[i] : v[i + 8];
+        a[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, 16);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool up = (lane & 8) != 0;
+        const float keep = up ? a[i + 4] : a[i], give = up ? a[i] : a[i + 4];
+        b[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, 8);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const bool up = (lane & 4) != 0;
+        const float keep = up ? b[i + 2] : b[i], give = up ? b[i] : b[i + 2];
+        c[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, 4);
+    }
+    const bool up = (lane & 2) != 0;
+    const float keep = up ? c[1] : c[0], give = up ? c[0] : c[1];
+    const float d = keep + __shfl_xor_sync(0xFFFFFFFFu, give, 2);
+    return d + __shfl_xor_sync(0xFFFFFFFFu, d, 1);
+}
+
 // ------------------------------------------------------------ the GEMM
 __global__ void __launch_bounds__(128, 1) gemm_kernel(const __grid_constant__ GemmArgs g)
 {
@@ -242,30 +298,27 @@ __global__ void __launch_bounds__(128, 1) gemm_kernel(const __grid_constant__ Ge
     if (ok) {
         const int64_t row = (int64_t)tile * kTileM + warp * 32 + lane;
         const bool valid = row < g.m_valid;
+        // a thread owns a row: 16 consecutive columns are four 16-byte accesses
+        // where the rows are 16-byte aligned
+        const bool fwide = ((reinterpret_cast<uintptr_t>(g.fout) | (uintptr_t)(g.ld_fout * 4)) & 15) == 0;
+        const bool zwide = ((reinterpret_cast<uintptr_t>(g.zin) | (uintptr_t)(g.N * 4)) & 15) == 0;
         for (int cl = 0; cl < nt; cl += 16) {
             const int c0 = n0 + cl;       // column of D
             float v[16];
             tmem_ld16(tmem_d + ((uint32_t)(warp * 32) << 16) + (uint32_t)cl, v);
-            if (g.epi == EPI_STORE_F32 || g.epi == EPI_LOGITS) {
-                if (valid) {
+            if (g.epi == EPI_HIDDEN_FWD || g.epi == EPI_LOGITS) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        g.fout[row * g.ld_fout + c0 + i] = v[i] + (g.epi == EPI_LOGITS ? g.bias[c0 + i] : 0.0f);
-                }
-            } else {
+                for (int i = 0; i < 16; ++i) v[i] = v[i] + g.bias[c0 + i];
+            }
+            if (g.epi != EPI_HIDDEN_BWD && valid) store16(g.fout + row * g.ld_fout + c0, v, fwide);
+            if (g.epi == EPI_HIDDEN_FWD || g.epi == EPI_HIDDEN_BWD) {
                 uint16_t h[16];
                 float dz[16];
+                if (g.epi == EPI_HIDDEN_BWD && valid) load16(g.zin + row * g.N + c0, dz, zwide);
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                    float y;
-                    if (g.epi == EPI_HIDDEN_FWD) {
-                        const float z = v[i] + g.bias[c0 + i];
-                        if (valid) g.fout[row * g.ld_fout + c0 + i] = z;
-                        y = gelu(z);
-                    } else {
-                        y = valid ? v[i] * gelu_grad(g.zin[row * g.N + c0 + i]) : 0.0f;
-                    }
-                    if (!valid) y = 0.0f;
+                    float y = 0.0f;
+                    if (valid) y = g.epi == EPI_HIDDEN_FWD ? gelu(v[i]) : v[i] * gelu_grad(dz[i]);
                     dz[i] = y;
                     h[i] = f2bf(y);
                 }
@@ -276,12 +329,8 @@ __global__ void __launch_bounds__(128, 1) gemm_kernel(const __grid_constant__ Ge
                         *reinterpret_cast<uint16_t *>(g.pkT_out + packed_offset(c0 + i, row, g.pkT_cols)) = h[i];
                 }
                 if (g.epi == EPI_HIDDEN_BWD && g.bias_grad) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        float s = dz[i];
-                        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-                        if (lane == 0) atomicAdd(&g.bias_grad[c0 + i], s);
-                    }
+                    const float s = column_sum16(dz, lane);
+                    if ((lane & 1) == 0) atomicAdd(&g.bias_grad[c0 + (lane >> 1)], s);
                 }
             }
         }
@@ -331,6 +380,21 @@ void set_wait_test(int withhold, uint32_t spin_limit)
     g_spin_limit = spin_limit;
 }
 
+// Columns of D per CTA.  The matrices are small: what a launch costs is one
+// CTA's chain of load, MMAs and epilogue, and the epilogue (GELU, the packed
+// and transposed stores) grows with the columns.  So 64 columns only where the
+// row tiles fill the GPU anyway, down to 16 where 64 would leave SMs idle
+// (1024 x 256 x 256 forward: 32 CTAs of 64 columns 16.4 us, 128 of 16
+// 7.2 us).  Other widths run as one column tile.
+static int column_tile(int N, int row_tiles)
+{
+    if (N < 128 || N % 64 != 0) return N;
+    constexpr int kFill = 128;   // CTAs that occupy most of the 152 SMs
+    for (int nt = 64; nt > 16; nt /= 2)
+        if (row_tiles * (N / nt) >= kFill) return nt;
+    return 16;
+}
+
 cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t s)
 {
     // Shared memory also caps how many CTAs share an SM: request enough that
@@ -338,7 +402,8 @@ cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t s)
     GemmArgs a = g;
     a.withhold = g_withhold;
     a.spin_limit = g_spin_limit;
-    a.ntile = (g.N >= 128 && g.N % 64 == 0) ? 64 : g.N;   // column tiles per row tile: N / ntile
+    const int tiles = (g.M + kTileM - 1) / kTileM;
+    a.ntile = column_tile(g.N, tiles);
     const int ncols = a.ntile <= 32 ? 32 : (a.ntile <= 64 ? 64 : (a.ntile <= 128 ? 128 : 256));
     const size_t per_sm = 233472, reserve = 1024;
     const size_t cap_ctas = (size_t)(512 / ncols);
@@ -350,7 +415,6 @@ cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t s)
     if (smem < floor_bytes) smem = floor_bytes;
     cudaError_t e = cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int tiles = (g.M + kTileM - 1) / kTileM;
     const dim3 grid((unsigned)tiles, (unsigned)(g.N / a.ntile));
     gemm_kernel<<<grid, 128, smem, s>>>(a);
     return cudaGetLastError();

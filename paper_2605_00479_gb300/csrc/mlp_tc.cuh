@@ -2,9 +2,9 @@
 //
 // D[M x N] (fp32, in tensor memory) = sum over K of A[M x K] * B[N x K]^T with
 // A and B in bf16.  One CTA of 128 threads owns a 128-row x ntile-column tile
-// of D (ntile = 64 when N >= 128 is a multiple of 64, else N; grid = row
-// tiles x column tiles); the accumulator occupies ntile columns of tensor
-// memory.
+// of D (ntile = 64, 32 or 16 when N >= 128 is a multiple of 64, by how many row
+// tiles there are, else N; grid = row tiles x column tiles); the accumulator
+// occupies ntile (at least 32) columns of tensor memory.
 //
 // Operands live in global memory in the "packed" layout that tcgen05 reads
 // without swizzling (K-major core matrices of 8 rows x 16 bytes):
