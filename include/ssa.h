@@ -332,8 +332,8 @@ int ssa_tail_stats(int64_t *moved, int64_t *lock_timeouts, int64_t *resumed);
  * kernels sort the parked trajectories by that prediction; the second launch
  * resumes them, largest first, so the launch ends on short ones.
  *   mode         0 off; 1 automatic (the default: when a0(x0) * t_end >= 4096
- *                events and there are at least 2 trajectories per resident
- *                lane, 2 * SMs * 1024); 2 always
+ *                events and there are at least 608 trajectories per SM, 2048
+ *                in fp64 and for batches); 2 always
  *   park_events  the parking point: 0 (the default) for a0(x0) * t_end / 5
  *                (at least 256), else an even number >= 2; no split when it
  *                is >= the run's max_events

@@ -75,7 +75,15 @@ int g_tail_lock_spins = 0;   // 0: the kernels' default bound
 int g_longest_first = 1;
 int64_t g_park_events = 0;
 constexpr double kLongestFirstMinEvents = 4096.0;   // estimated events per trajectory
-constexpr int64_t kLongestFirstMinPerLane = 2;      // trajectories per resident lane
+// trajectories per multiprocessor: batches and fp64, single runs of the other
+// modes.  Schloegl, unsplit -> split, ms: mixed bf16 8 10^4 28.9 -> 30.1, 10^5
+// 32.2 -> 25.3, 2 10^5 38.0 -> 34.6, 3 10^5 52.6 -> 45.6; uniform f16 SR 1.5 10^5
+// 83.6 -> 74.3; uniform f16 RN 10^5 83.3 -> 62.0; repressilator 10^5 and below
+// unchanged.  fp64 6 10^4 420 -> 662: a warp of long trajectories holds its
+// scheduler's binary64 unit.  A sweep of three models x 500 sets x 64
+// trajectories 158 -> 238.
+constexpr int64_t kLongestFirstMinPerSM = 2048;
+constexpr int64_t kLongestFirstMinPerSM32 = 608;
 constexpr double kLongestFirstMinSpread = 4.0;      // batches: largest / smallest estimate over the sets
 std::atomic<long long> g_direct_launches{0};        // kernels launched by launch_run
 
@@ -330,10 +338,10 @@ ssa::OrderModel order_model(const ssa::RunArgs &a, const ssa::LongestFirstScratc
 // Whether a single-queue run is split into park / order / resume, and with
 // which parking point; returns the scratch (null: one plain launch).  The
 // split pays when trajectories are long (the end of a persistent launch waits
-// for the trajectories that started last) and every lane runs several.  A
+// for the trajectories that started last) and there are enough of them.  A
 // failed allocation falls back to the plain launch.
-char *plan_longest_first(const ssa_model &m, const int32_t *x0, int normalise, double t_end, int64_t n_work,
-                         int64_t max_events, cudaStream_t s, int64_t *park)
+char *plan_longest_first(const ssa_model &m, const int32_t *x0, int normalise, int precision, double t_end,
+                         int64_t n_work, int64_t max_events, cudaStream_t s, int64_t *park)
 {
     if (g_longest_first == 0 || n_work < 1) return nullptr;
     const double est = estimated_events(m, x0, normalise, t_end);
@@ -348,7 +356,8 @@ char *plan_longest_first(const ssa_model &m, const int32_t *x0, int normalise, d
         int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return nullptr;
-        if (!(est >= kLongestFirstMinEvents) || n_work < kLongestFirstMinPerLane * (int64_t)sms * 1024) return nullptr;
+        const int64_t per_sm = precision == SSA_FP64 ? kLongestFirstMinPerSM : kLongestFirstMinPerSM32;
+        if (!(est >= kLongestFirstMinEvents) || n_work < per_sm * (int64_t)sms) return nullptr;
     }
     char *p = nullptr;
     if (cudaMallocAsync(reinterpret_cast<void **>(&p), longest_first_bytes(n_work, m.N), s) != cudaSuccess) {
@@ -413,7 +422,7 @@ int launch_run(const ssa_model *model, int64_t n_work, int64_t stride, uint64_t 
     const int norm = normalise ? 1 : 0;
     const ssa::Launcher launch = launcher_for(model->family);
     int64_t park = 0;
-    char *scratch = plan_longest_first(*model, x0, normalise, t_end, n_work, max_events, s, &park);
+    char *scratch = plan_longest_first(*model, x0, normalise, precision, t_end, n_work, max_events, s, &park);
     if (scratch) {
         // launch 1: every trajectory up to `park` events; the unfinished are parked
         ssa::LongestFirstScratch L = carve_longest_first(scratch, n_work, model->N);
@@ -1098,7 +1107,7 @@ int ssa_batch_create(int n_groups, const ssa_batch_group *groups, double t_end, 
         int dev = 0, sms = 0;
         const bool ok = cudaGetDevice(&dev) == cudaSuccess &&
                         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
-        const bool enough = g_longest_first == 2 || (ok && work >= kLongestFirstMinPerLane * (int64_t)sms * 1024);
+        const bool enough = g_longest_first == 2 || (ok && work >= kLongestFirstMinPerSM * (int64_t)sms);
         for (int g = 0; g < n_groups && enough; ++g) {
             const int64_t items = groups[g].n_sets * groups[g].traj_per_set;
             if (items < 1) continue;
