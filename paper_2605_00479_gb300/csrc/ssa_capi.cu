@@ -152,6 +152,8 @@ ssa::Launcher launcher_for(int family)
 
 bool finite_double(double v) { return std::isfinite(v); }
 
+size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
 // c'_j = c_j / prod_i r_ij!, then (normalise) times the falling factorials of
 // the constant species' counts, species ascending, factor m ascending; all in
 // binary64 (reading of Sec. 4.2: k1 A and k3 B formed before rounding).
@@ -815,7 +817,9 @@ int ssa_rdme_run(const ssa_model *model, int nx, int ny, int nz, const double *d
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t lat_bytes = sizeof(int32_t) * (size_t)S * (size_t)N;
     char *d = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&d), 256 + lat_bytes, s);
+    const size_t table_at = align_up(256 + lat_bytes, 256);   // VoxelTable rows of the kernels that read them
+    const size_t table_bytes = (size_t)ssa::kTableRows * 8 * (size_t)elem;
+    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&d), table_at + table_bytes, s);
     if (e != cudaSuccess) {
         delete A;
         return e == cudaErrorMemoryAllocation ? fail(SSA_ENOMEM, "RDME tables: out of device memory")
@@ -823,6 +827,7 @@ int ssa_rdme_run(const ssa_model *model, int nx, int ny, int nz, const double *d
     }
     A->a.queue_head = reinterpret_cast<unsigned long long *>(d);
     A->x0_lat = reinterpret_cast<const int32_t *>(d + 256);
+    A->table = d + table_at;
     e = cudaMemsetAsync(d, 0, sizeof(unsigned long long), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d + 256, x0, lat_bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) {
@@ -933,8 +938,6 @@ struct ssa_batch {
 };
 
 namespace {
-
-size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Device bytes of one group's per-set tables: c' [S][M] f64, Hill amplitudes
 // [S][M][2] f64, x0 [S][N] i32, each 256-byte aligned.  Used both to size
