@@ -203,7 +203,8 @@ __device__ inline int64_t first_leap_after(double s, double tau)
 //      rejection round an iteration, so lanes wait only for the largest total
 //      of a lane, not for the largest of every channel.
 // Quantities that only the slow test reads are computed only there.  Measured (GB300, Schloegl fp32, 1.5 10^5 trajectories,
-// 2000 leaps): 51.1 -> 28.4 ms.
+// 2000 leaps): 51.1 -> 28.4 ms, 23.5 ms with the slow test decided by hardware
+// logarithms (Rejection::settle).
 template <class R>
 struct SamplerMath;
 template <>
@@ -277,9 +278,39 @@ struct Rejection {
         }
         return false;
     }
+    // The binary32 test decides by hardware logarithms first.  Both sides of the
+    // inequality consist of terms of size up to `size`; the contract's operations
+    // err by less than 2^-20 of it, the approximate ones (lg2.approx: 2^-22
+    // absolute in log2) by less than 2^-19, so a difference beyond 2^-17 of it
+    // has the contract's sign.  What lies closer (0.2% of the tests at lambda =
+    // 20), and lambda above 2000, where the margin would settle little, is
+    // evaluated as the contract says.
+    __device__ __forceinline__ int settle(float lam, float us, float V, float kf, const float *small) const
+    {
+        auto ln = [](float x) {
+            float y;
+            asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+            return y * 0.693147181f;
+        };
+        const float invalpha = __fmaf_rn(1.1328f, rcp_seed((float)b - 3.4f), 1.1239f);
+        const float edge = __fmaf_rn((float)a, rcp_seed(us * us), (float)b);
+        const float lhs = ln(V * invalpha) - ln(edge);
+        const float x = kf + 1.0f;
+        const float llam = kf * ln(lam), lx = (x - 0.5f) * ln(x);
+        const float fact = kf < 10.0f ? small[(int)kf] : lx - x + 0.918938533f + 0.0833333333f * rcp_seed(x);
+        const float d = (llam - lam - fact) - lhs;
+        const float size = lam + llam + lx + x + 64.0f;
+        return fabsf(d) > size * 0x1p-17f ? (d > 0.0f ? 1 : -1) : 0;
+    }
     __device__ __forceinline__ bool slow(R lam, R us, R V, R kf, const R *small) const
     {
         using Q = SamplerMath<R>;
+        if constexpr (sizeof(R) == 4) {
+            if (lam < 2000.0f) {
+                const int sign = settle(lam, us, V, kf, small);
+                if (sign != 0) return sign > 0;
+            }
+        }
         const R invalpha = R(sizeof(R) == 8 ? 1.1239 : 1.1239f) +
                            Q::div(R(sizeof(R) == 8 ? 1.1328 : 1.1328f), b - R(sizeof(R) == 8 ? 3.4 : 3.4f));
         R lhs = Q::log(V) + Q::log(invalpha);

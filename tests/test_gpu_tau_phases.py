@@ -61,3 +61,11 @@ def test_block_sizes(ssa, block):
         both(ssa, P.repressilator(h=3), P.REPRESSILATOR_X0, 301, 2.0, 0.02, [1.0, 2.0], "mixed_f16", "sr", seed=4)
     finally:
         ssa.set_launch_config()
+
+
+@pytest.mark.parametrize("lam", [10.0, 11.3, 14.0, 20.0, 47.0, 150.0, 1000.0, 1999.0, 2500.0])
+def test_many_draws_of_the_rejection_method(ssa, lam):
+    # every acceptance decision of 2^18 draws: the approximate test must never
+    # decide differently from the contract's
+    md = {"order": np.array([[0]], np.int32), "stoich": np.array([[1]], np.int32), "rate": np.array([lam])}
+    both(ssa, md, [0], 2**16, 4.0, 1.0, [1.0, 2.0, 3.0, 4.0], "fp32", "rn", seed=9)
