@@ -128,12 +128,15 @@ cudaError_t launch_family(const RunArgs &a, int prec, int sr, LaunchConfig cfg, 
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    // dynamic shared memory: the columns of a general network's lanes (at most 41 KB)
+    // dynamic shared memory: the columns of a general network's lanes.  The
+    // attribute gets the same value (the largest, 41 KB) on every call, so calls
+    // from several threads do not lower it for each other.
     auto columns = [&](int b) -> size_t {
         return std::is_same<ModelF, GeneralModel>::value && a.n_sets == 1 ? general_columns(a.N, a.M, prec, b) : 0;
     };
     if (columns(256) > 0) {
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)columns(256));
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)general_columns(kMaxN, kMaxM, prec, 256));
         if (e != cudaSuccess) return e;
     }
     int block = cfg.block;

@@ -213,11 +213,13 @@ int device_sms(int *sms)
     return cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
 }
 
-// Launch of a histogram kernel with its block-private counters.
+// Launch of a histogram kernel with its block-private counters (the attribute
+// always gets the largest size, so concurrent calls do not lower it).
 template <class Kernel, class... Args>
 int launch_histogram(Kernel k, int64_t grid, size_t bytes, cudaStream_t s, Args... args)
 {
-    if (bytes > 48 * 1024 && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+    if (bytes > 48 * 1024 &&
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedWords * 4) != cudaSuccess)
         return SSA_ECUDA;
     k<<<(unsigned)grid, kThreads, bytes, s>>>(args...);
     return cudaGetLastError() == cudaSuccess ? SSA_OK : SSA_ECUDA;

@@ -598,9 +598,11 @@ cudaError_t tau_launch_model(const RunArgs &a, int prec, int sr, int block, int 
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    // at most 16 channels x 256 threads x 3 binary64 values + 4 KB: 100 KB
+    // The attribute gets the same value on every call (the largest a launch can
+    // ask for, 100 KB), so calls from several threads do not lower it for each other.
     const size_t smem = tau_shared_bytes(a, block, prec == FP64 ? 8 : 4);
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr int kMost = kMaxK * 4 + 3 * kMaxM * 256 * 8;
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem);
     if (e != cudaSuccess) return e;
