@@ -77,19 +77,21 @@ def workload():
 # Algorithmic 32-bit operations per event for the Schloegl structure with the
 # reservoirs folded (chains: X(X-1) in reaction 1, X(X-1)(X-2) in reaction 2,
 # X in reaction 4; reaction 3 is a constant).  Counted from the method:
-#   Philox4x32-10 block: 10 rounds x (2 mul-hi + 2 mul-lo + 4 xor + 2 add) = 100
+#   Philox4x32-10 block: 18 32x32->64-bit multiplications (two of the twenty
+#   depend on the trajectory alone) + 19 three-input xors = 37
 #   uniforms: half a block per step (two steps per block) + 2 x 4 to scale
 #   log: 25 (exponent split 6, s = (m-1)/(m+1) 3, z and series 8, recombine 8)
 #   tau division, target multiply, clock add: 3
 #   mass-action factor: subtract, convert, multiply = 3 (+2 roundings in 16 bit)
 #   partial sums: M - 1 adds (+ M - 1 roundings in uniform mode)
 #   selection M compares + branch 2, update 2, snapshot compare 1, loop 4
+PHILOX_OPS = 37
 SCHLOGL_FACTORS = 6  # X(X-1): 2, X(X-1)(X-2): 3, X: 1
 M_REACTIONS = 4
 
 
 def ops_per_event(prec, rnd):
-    philox = 100
+    philox = PHILOX_OPS
     ops = philox * 0.5 + 8 + 25 + 3
     ops += SCHLOGL_FACTORS * 3
     ops += (M_REACTIONS - 1)
@@ -125,7 +127,7 @@ NCU_TRAFFIC_PER_TRAJ = {
 def device_source_hash():
     import hashlib
     h = hashlib.sha256()
-    for f in ("ssa_device.cuh", "ssa_models.h", "ssa_launch.h", "ssa_order.cu"):
+    for f in ("ssa_device.cuh", "ssa_fast.cuh", "ssa_general.cuh", "ssa_models.h", "ssa_launch.h", "ssa_order.cu"):
         with open(os.path.join(ROOT, "paper_2605_00479_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -892,16 +894,16 @@ def model_ops_per_event(md, prec, rnd, normalise=False):
             factors += f
             chain16 += 2 * f
     n_update = int(sum(1 for i in range(N) if not const[i])) + 1
-    ops = 100 * 0.5 + 8 + 25 + 3 + 3 * factors + hill_ops + (M - 1) + M + 2 + n_update + 1 + 4
+    ops = PHILOX_OPS * 0.5 + 8 + 25 + 3 + 3 * factors + hill_ops + (M - 1) + M + 2 + n_update + 1 + 4
     if prec.startswith(("mixed", "uniform")):
         ops += chain16                      # one conversion per rounded chain operation
     if prec.startswith("uniform"):
         ops += (M - 1 + 5) * 2
     if rnd == "sr":
         n_sr = chain16 + (M - 1 + 5 if prec.startswith("uniform") else 0)
-        ops += 100 * ((n_sr + 7) // 8)
+        ops += PHILOX_OPS * ((n_sr + 7) // 8)
     if rnd == "sra":
-        ops += 100 * ((M + 7) // 8)
+        ops += PHILOX_OPS * ((M + 7) // 8)
     return float(ops)
 
 
