@@ -116,10 +116,10 @@ def ops_per_event(prec, rnd):
 # includes a hash of the device code, and a changed kernel reports null.
 NCU_TRAFFIC_PER_TRAJ = {
     # mixed_bf16 RN (the headline kernel), 4e5 trajectories, snapshots of X only,
-    # default launch shape, longest-first split: launch 1 13,282,304 R +
-    # 13,166,848 W; ordering kernels 10,457,088 R; launch 2 87,435,776 R +
-    # 85,055,232 W
-    ("6501ac81666e509f", "mixed_bf16:rn"): (13282304 + 13166848 + 5229056 + 8448 + 5219584 + 87435776 + 85055232)
+    # default launch shape, longest-first split: launch 1 13,147,648 R +
+    # 12,972,544 W; ordering kernels 10,457,344 R; launch 2 84,285,952 R +
+    # 84,645,888 W
+    ("e7dfc8f7b0080e12", "mixed_bf16:rn"): (13147648 + 12972544 + 5228800 + 8448 + 5220096 + 84285952 + 84645888)
     / 400000,
 }
 
@@ -585,16 +585,16 @@ RDME_CAP = 4_000_000
 # hash, workload, mode); a changed kernel reports null until re-counted.
 NCU_PER_UNIT = {
     # tau, 2e5 trajectories, one launch per mode (compiled Schloegl structure)
-    ("3c23ba7ec014e430", "tau", "fp32:rn"): {"warp_inst": 6.2743, "dram_bytes": 0.01304},
-    ("3c23ba7ec014e430", "tau", "mixed_f16:rn"): {"warp_inst": 6.3621, "dram_bytes": 0.01402},
-    ("3c23ba7ec014e430", "tau", "mixed_bf16:rn"): {"warp_inst": 6.2441, "dram_bytes": 0.01384},
-    ("3c23ba7ec014e430", "tau", "uniform_f16:sr"): {"warp_inst": 6.5411, "dram_bytes": 0.01409},
-    ("3c23ba7ec014e430", "tau", "uniform_bf16:sr"): {"warp_inst": 6.4396, "dram_bytes": 0.01364},
+    ("2c464a8e963606ca", "tau", "fp32:rn"): {"warp_inst": 2.8639, "dram_bytes": 0.00734},
+    ("2c464a8e963606ca", "tau", "mixed_f16:rn"): {"warp_inst": 2.9236, "dram_bytes": 0.00712},
+    ("2c464a8e963606ca", "tau", "mixed_bf16:rn"): {"warp_inst": 2.8484, "dram_bytes": 0.00725},
+    ("2c464a8e963606ca", "tau", "uniform_f16:sr"): {"warp_inst": 2.9542, "dram_bytes": 0.00747},
+    ("2c464a8e963606ca", "tau", "uniform_bf16:sr"): {"warp_inst": 2.8884, "dram_bytes": 0.00708},
     # rdme, 32768 lattices, one launch per mode
-    ("1a5bb4191f753f15", "rdme", "fp32:rn"): {"warp_inst": 30.1687, "dram_bytes": 0.00014},
-    ("1a5bb4191f753f15", "rdme", "mixed_f16:rn"): {"warp_inst": 32.4930, "dram_bytes": 0.00017},
-    ("1a5bb4191f753f15", "rdme", "mixed_bf16:rn"): {"warp_inst": 32.5187, "dram_bytes": 0.00063},
-    ("1a5bb4191f753f15", "rdme", "mixed_f16:sr"): {"warp_inst": 43.9234, "dram_bytes": 0.00106},
+    ("24bc6759fdb0d3cf", "rdme", "fp32:rn"): {"warp_inst": 22.8227, "dram_bytes": 0.00003},
+    ("24bc6759fdb0d3cf", "rdme", "mixed_f16:rn"): {"warp_inst": 22.7984, "dram_bytes": 0.00022},
+    ("24bc6759fdb0d3cf", "rdme", "mixed_bf16:rn"): {"warp_inst": 22.8370, "dram_bytes": 0.00069},
+    ("24bc6759fdb0d3cf", "rdme", "mixed_f16:sr"): {"warp_inst": 36.5527, "dram_bytes": 0.00110},
 }
 
 
