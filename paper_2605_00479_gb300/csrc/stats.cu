@@ -37,9 +37,15 @@ constexpr int kSharedWords = 16384;
 constexpr int kThreads = 512;
 constexpr int kBlocksPerSM = 2;
 
-int histogram_copies(int bins)
+// Few values: clearing and adding up the copies would cost more than the
+// counts that meet in one (int32 counts, GB300 kernel time: 1001 in 1024 bins
+// 2.6 us with the copies, 2.2 with one; 30001 in 251 bins 2.7 and 2.1).
+constexpr int64_t kFewValues = 65536;
+
+int histogram_copies(int bins, int64_t n)
 {
     if (bins > kSharedBins) return 0;
+    if (n < kFewValues) return 1;
     int c = 32;
     while (c > 1 && (int64_t)c * (bins | 1) > kSharedWords) c /= 2;
     return c;
@@ -56,6 +62,17 @@ __device__ __forceinline__ void clear_shared(unsigned int *sh, int bins, int cop
 __device__ __forceinline__ void flush_shared(const unsigned int *sh, int bins, int copies, unsigned long long *hist)
 {
     __syncthreads();
+    if (copies == 1) {   // four reads in flight (1001 counts in 8192 bins: 4.4 -> 2.8 us)
+        for (int k = threadIdx.x; k < bins; k += 4 * blockDim.x) {
+            unsigned int t[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) t[i] = k + i * (int)blockDim.x < bins ? sh[k + i * (int)blockDim.x] : 0u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (t[i]) atomicAdd(&hist[k + i * (int)blockDim.x], (unsigned long long)t[i]);
+        }
+        return;
+    }
     for (int k = threadIdx.x; k < bins; k += blockDim.x) {
         unsigned int t = 0;
         for (int c = 0; c < copies; ++c) t += sh[c * (bins | 1) + k];
@@ -238,9 +255,10 @@ int ssa_count_histogram(const void *values, int elem_bytes, int64_t n, int bins,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int sms = 0;
     if (!device_sms(&sms)) return SSA_ECUDA;
-    int64_t grid = (n + kThreads * 8 - 1) / (kThreads * 8);
+    const int64_t per_block = n < kFewValues ? kThreads * 4 : kThreads * 8;
+    int64_t grid = (n + per_block - 1) / per_block;
     if (grid > (int64_t)sms * kBlocksPerSM) grid = (int64_t)sms * kBlocksPerSM;
-    const int copies = histogram_copies(bins);
+    const int copies = histogram_copies(bins, n);
     auto *h = reinterpret_cast<unsigned long long *>(hist);
     auto *c = reinterpret_cast<unsigned long long *>(n_clamped);
     const size_t bytes = histogram_bytes(bins, copies);
@@ -270,7 +288,7 @@ int ssa_dwell_histogram(const void *series, int elem_bytes, int K, int64_t n, in
     if (!device_sms(&sms)) return SSA_ECUDA;
     int64_t grid = (n + kThreads - 1) / kThreads;
     if (grid > (int64_t)sms * 4) grid = (int64_t)sms * 4;
-    const int copies = histogram_copies(K);
+    const int copies = histogram_copies(K, n * K);
     auto *h = reinterpret_cast<unsigned long long *>(hist);
     const size_t bytes = histogram_bytes(K, copies);
     if (elem_bytes == 4)

@@ -21,7 +21,7 @@ def ssa():
 
 @pytest.mark.parametrize("dtype", [np.int32, np.int16])
 @pytest.mark.parametrize("bins", [1, 2, 512, 8192, 8193])
-@pytest.mark.parametrize("n", [1, 3, 7, 8, 9, 4097, 1000003])
+@pytest.mark.parametrize("n", [1, 3, 7, 8, 9, 4097, 65535, 65536, 1000003])
 @pytest.mark.parametrize("skip", [0, 1, 3, 7])
 def test_count_histogram(ssa, dtype, bins, n, skip):
     rng = np.random.default_rng(n + bins + skip)
