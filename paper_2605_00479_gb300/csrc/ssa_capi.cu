@@ -116,11 +116,10 @@ bool matches(const ssa_model &m)
         if ((m.constant[i] != 0) != (S::cs[i] != 0)) return false;
     for (int j = 0; j < S::M; ++j) {
         if (m.law[j] != S::lw[j]) return false;
-        if (S::lw[j] == SSA_LAW_HILL_REPRESSION) {
-            if ((int)m.hill[j][2] != S::hh[j] || (int)m.hill[j][3] != S::hreg[j]) return false;
-            continue;
-        }
-        for (int i = 0; i < S::N; ++i) {
+        if (S::lw[j] == SSA_LAW_HILL_REPRESSION &&
+            ((int)m.hill[j][2] != S::hh[j] || (int)m.hill[j][3] != S::hreg[j]))
+            return false;
+        for (int i = 0; i < S::N; ++i) {   // Hill rows have no reactants (order 0 on both sides)
             if (m.order[j][i] != S::ord[j][i]) return false;
             if (!S::cs[i] && m.stoich[j][i] != S::nu[j][i]) return false;
         }
