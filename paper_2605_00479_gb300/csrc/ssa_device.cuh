@@ -963,8 +963,9 @@ __device__ __forceinline__ void general_propensities(const RunArgs &a, const Lan
 // ------------------------------------------------- one step, general model
 // Same contract as ssa_step, with the structure read from the kernel
 // arguments in runtime loops (state and tables in local memory).  Used for
-// networks that match no compiled structure.
-template <int PREC, int SR>
+// networks that match no compiled structure.  INLINE: snapshots unrolled in
+// place instead of out of line.
+template <int PREC, int SR, bool INLINE>
 __device__ __noinline__ void ssa_step_general(const RunArgs &a, Lane<GeneralModel, PREC> &L, uint32_t w0, uint32_t w1,
                                               const typename ModeTraits<PREC>::P *smp,
                                               typename ModeTraits<PREC>::P t_end)
@@ -972,6 +973,10 @@ __device__ __noinline__ void ssa_step_general(const RunArgs &a, Lane<GeneralMode
     using Tr = ModeTraits<PREC>;
     using P = typename Tr::P;
     const P kInf = P(__int_as_float(0x7F800000));
+    auto end = [&]() {
+        if constexpr (INLINE) finish<GeneralModel, PREC>(a, L);
+        else finish_general<PREC>(a, L);
+    };
 
     if (L.n >= a.max_events) {
         if (a.parked && L.n < a.cap_events) {
@@ -979,7 +984,7 @@ __device__ __noinline__ void ssa_step_general(const RunArgs &a, Lane<GeneralMode
             return;
         }
         L.status |= ST_MAX_EVENTS;
-        finish_general<PREC>(a, L);
+        end();
         return;
     }
     Rounder<PREC, SR> R;
@@ -1007,9 +1012,9 @@ __device__ __noinline__ void ssa_step_general(const RunArgs &a, Lane<GeneralMode
         }
     }
     const P a0 = S[a.M - 1];
-    if (is_nan<PREC>(a0)) { L.status |= ST_NAN; finish_general<PREC>(a, L); return; }
-    if (a0 == kInf) { L.status |= ST_OVERFLOW; finish_general<PREC>(a, L); return; }
-    if (a0 == P(0)) { finish_general<PREC>(a, L); return; }
+    if (is_nan<PREC>(a0)) { L.status |= ST_NAN; end(); return; }
+    if (a0 == kInf) { L.status |= ST_OVERFLOW; end(); return; }
+    if (a0 == P(0)) { end(); return; }
 
     P tau, target, t_new;
     if constexpr (Tr::kF64) {
@@ -1037,11 +1042,12 @@ __device__ __noinline__ void ssa_step_general(const RunArgs &a, Lane<GeneralMode
         }
     }
     while (L.s_next < t_new) {
-        L.status = store_state_loop<GeneralModel>(a, L.k, L.item, L.x, L.status);
+        if constexpr (INLINE) store_state<GeneralModel>(a, L.k, L.item, L.x, L.status);
+        else L.status = store_state_loop<GeneralModel>(a, L.k, L.item, L.x, L.status);
         L.k += 1;
         L.s_next = L.k < a.K ? smp[L.k] : kInf;
     }
-    if (t_new > t_end) { finish_general<PREC>(a, L); return; }
+    if (t_new > t_end) { end(); return; }
 
     int mu = -1;
 #pragma unroll 1
@@ -1062,7 +1068,7 @@ __device__ __noinline__ void ssa_step_general(const RunArgs &a, Lane<GeneralMode
     L.n += 1;
     if (negative) {
         L.status |= ST_STATE_RANGE;
-        finish_general<PREC>(a, L);
+        end();
     }
 }
 
@@ -1274,7 +1280,7 @@ __device__ __forceinline__ bool pool_visit(const RunArgs &a, TailPool<Model, PRE
 // trajectories to each other once the queue has drained (tail compaction,
 // above).  Returns once the warp has no more work, so the caller may move the
 // whole warp to another queue.
-template <class Model, int PREC, int SR>
+template <class Model, int PREC, int SR, bool INLINE = false>
 __device__ __forceinline__ void run_queue(const RunArgs &a, const typename ModeTraits<PREC>::P *smp,
                                           typename ModeTraits<PREC>::P t_end,
                                           TailPool<Model, PREC> *pool = nullptr)
@@ -1313,8 +1319,8 @@ __device__ __forceinline__ void run_queue(const RunArgs &a, const typename ModeT
             const uint64_t blk = (uint64_t)(L.n >> 1);
             const uint4 u = philox4x32_10(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), L.traj, 0u), a.key0, a.key1);
             if constexpr (std::is_same<Model, GeneralModel>::value) {
-                if (L.active) ssa_step_general<PREC, SR>(a, L, u.x, u.y, smp, t_end);
-                if (L.active) ssa_step_general<PREC, SR>(a, L, u.z, u.w, smp, t_end);
+                if (L.active) ssa_step_general<PREC, SR, INLINE>(a, L, u.x, u.y, smp, t_end);
+                if (L.active) ssa_step_general<PREC, SR, INLINE>(a, L, u.z, u.w, smp, t_end);
             } else {
                 if (L.active) ssa_step<Model, PREC, SR>(a, L, u.x, u.y, smp, t_end);
                 if (L.active) ssa_step<Model, PREC, SR>(a, L, u.z, u.w, smp, t_end);
@@ -1341,32 +1347,36 @@ __device__ __forceinline__ void run_any(const RunArgs &a, const typename ModeTra
     else run_queue_fast<Model, PREC, SR>(a, smp, t_end, ln2, pool);
 }
 
-// Single-model launches: the structure lists of a general network.  A launch
-// over several parameter sets of one keeps ssa_step_general (its constants
-// differ from lane to lane).
-template <class Model, int PREC>
+// Single-model launches.  General networks: the structure lists, or with PLAIN
+// ssa_step_general for every step (general_plain says when), in a kernel of its
+// own because the register budget and the columns that serve the lists cost it
+// up to a third.  Its snapshots lie inline where the step rounds stochastically
+// and out of line elsewhere (uniform f16 SR 10% slower out of line, fp32 3% faster;
+// round to nearest then takes 64 registers, 8 bytes spilled).  Sweeps of 64 sets x
+// 1500 trajectories of a six-reaction network, in the lists' kernel -> in its own:
+// fp32 63.5 -> 50.1 ms, mixed bf16 SR 107.4 -> 65.6, uniform f16 SR 109.8 -> 77.1;
+// 20000 trajectories of a network with a change of 2000, fp32 13.0 -> 10.3 ms,
+// uniform f16 SR 28.9 -> 21.3.
+template <class Model, int PREC, bool PLAIN>
 struct KernelTables {
     using type = int;
 };
 template <int PREC>
-struct KernelTables<GeneralModel, PREC> {
+struct KernelTables<GeneralModel, PREC, false> {
     using type = GeneralTables<PREC>;
 };
 
-template <class Model, int PREC, int SR>
+template <class Model, int PREC, int SR, bool PLAIN>
 __device__ __forceinline__ void run_single(const RunArgs &a, const typename ModeTraits<PREC>::P *smp,
                                            typename ModeTraits<PREC>::P t_end, const double2 *ln2,
-                                           const typename KernelTables<Model, PREC>::type *tables,
+                                           const typename KernelTables<Model, PREC, PLAIN>::type *tables,
                                            TailPool<Model, PREC> *pool)
 {
     extern __shared__ __align__(16) unsigned char columns[];   // general_columns bytes
-    if constexpr (std::is_same<Model, GeneralModel>::value) {
-        if (a.n_sets == 1) {
-            run_queue_general<PREC, SR>(a, smp, t_end, ln2, *tables, columns, pool);
-            return;
-        }
-    }
-    run_any<Model, PREC, SR>(a, smp, t_end, ln2, pool);
+    if constexpr (PLAIN) run_queue<Model, PREC, SR, SR == 1>(a, smp, t_end, pool);
+    else if constexpr (std::is_same<Model, GeneralModel>::value)
+        run_queue_general<PREC, SR>(a, smp, t_end, ln2, *tables, columns, pool);
+    else run_any<Model, PREC, SR>(a, smp, t_end, ln2, pool);
 }
 
 template <int PREC>
@@ -1381,8 +1391,9 @@ __device__ __forceinline__ void load_samples(const double *samples, int K, typen
 
 // ------------------------------------------------------------- the kernels
 // One model, one queue: arguments in parameter space.
-template <class Model, int PREC, int SR>
-__global__ void __launch_bounds__(256, (KernelMinBlocks<Model, PREC, SR>::value)) ssa_kernel(const __grid_constant__ RunArgs a)
+template <class Model, int PREC, int SR, bool PLAIN = false>
+__global__ void __launch_bounds__(256, (PLAIN ? (SR == 0 && PREC != FP64 ? 4 : 1) : KernelMinBlocks<Model, PREC, SR>::value))
+    ssa_kernel(const __grid_constant__ RunArgs a)
 {
     using P = typename ModeTraits<PREC>::P;
     __shared__ P smp[kMaxK];
@@ -1391,10 +1402,10 @@ __global__ void __launch_bounds__(256, (KernelMinBlocks<Model, PREC, SR>::value)
     const bool pooled = a.tail_stats != nullptr;
     if (pooled) pool_init(&pool);
     load_samples<PREC>(a.samples, a.K, smp, ln2);   // ends with __syncthreads
-    __shared__ typename KernelTables<Model, PREC>::type tables;
-    if constexpr (std::is_same<Model, GeneralModel>::value) build_general_tables<PREC>(a, &tables);
+    __shared__ typename KernelTables<Model, PREC, PLAIN>::type tables;
+    if constexpr (std::is_same<Model, GeneralModel>::value && !PLAIN) build_general_tables<PREC>(a, &tables);
     for (int pass = 0;; ++pass) {
-        run_single<Model, PREC, SR>(a, smp, to_time<PREC>(a.t_end), ln2, &tables, pooled ? &pool : nullptr);
+        run_single<Model, PREC, SR, PLAIN>(a, smp, to_time<PREC>(a.t_end), ln2, &tables, pooled ? &pool : nullptr);
         if (!pooled || pass > 0) break;
         // every warp has left the loop: records stranded by a lock wait that
         // gave up are resumed by warp 0 (the pool no longer changes)

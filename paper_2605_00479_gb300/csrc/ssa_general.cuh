@@ -9,7 +9,8 @@
 // columns of shared memory (word index * blockDim + thread: no bank
 // conflicts, and the lists' indices are the same for the whole warp).  The
 // arithmetic and its shortcuts are those of ssa_fast.cuh; steps outside that
-// domain run ssa_step_general.  Measured (GB300, six reactions, three species,
+// domain run ssa_step_general, and runs that start outside it (general_plain)
+// a kernel of their own.  Measured (GB300, six reactions, three species,
 // 10^5 trajectories to t = 50, fp32): 48.8 -> 23.8 ms;
 // repressilator with Hill exponent 3 (10^5, t = 5, mixed f16) 135.9 -> 40.9 ms.
 #pragma once
@@ -37,7 +38,6 @@ struct GeneralTables {
     int n_chg[kMaxM];
     P c[kMaxM], h0[kMaxM], h1[kMaxM];
     int max_chg;
-    int odd;                           // a Hill amplitude outside the fast division's range
     int moving;                        // bit i: species i changes or is read
 };
 
@@ -48,7 +48,6 @@ __device__ __forceinline__ void build_general_tables(const RunArgs &a, GeneralTa
     const int bd = (int)blockDim.x;
     if (threadIdx.x == 0) {
         T->max_chg = 0;
-        T->odd = 0;
         T->moving = 0;
         int n = 0;
         for (int j = 0; j < a.M; ++j) {
@@ -62,8 +61,6 @@ __device__ __forceinline__ void build_general_tables(const RunArgs &a, GeneralTa
                 T->h0[j] = to_prop<PREC>(a.hill_a0[j]);
                 T->h1[j] = to_prop<PREC>(a.hill_a[j]);
                 T->moving |= 1 << a.hill_reg[j];
-                if (ModeTraits<PREC>::k16 && T->h1[j] != P(0) && !(T->h1[j] >= P(0x1p-30f) && T->h1[j] <= P(0x1p31f)))
-                    T->odd = 1;
             } else {
                 for (int i = 0; i < a.N; ++i) {
                     if (a.order[j][i] == 0 || a.folded[j][i]) continue;
@@ -82,8 +79,6 @@ __device__ __forceinline__ void build_general_tables(const RunArgs &a, GeneralTa
                 T->moving |= 1 << i;
                 T->chg[j][c].offset = i * bd;
                 T->chg[j][c].nu = (float)a.stoich[j][i];
-                // counts stay below 2^23 + 64 * 2 * |nu|: exact only for small changes
-                if (a.stoich[j][i] > 1024 || a.stoich[j][i] < -1024) T->odd = 1;
                 c += 1;
             }
             T->n_chg[j] = c;
@@ -97,6 +92,31 @@ __device__ __forceinline__ void build_general_tables(const RunArgs &a, GeneralTa
 __host__ __device__ inline size_t general_columns(int N, int M, int prec, int block)
 {
     return (size_t)block * ((size_t)N * 4 + (size_t)M * (prec == FP64 || prec >= UNIFORM_F16 ? 8 : 4));
+}
+
+// Runs that go to the kernel without lists (PLAIN in ssa_device.cuh,
+// ssa_step_general for every step): several parameter sets (the lists hold one),
+// and one set where run_queue_general's steps would leave its domain anyway --
+// changes above 1024 (counts stay below 2^23 + 64 * 2 * |nu| within a slice, and
+// must stay exact in binary32), a moving or reactant count that starts at 2^23 or
+// more, and in the 16-bit modes a Hill amplitude that, rounded to the format, is
+// neither zero nor in [2^-30, 2^31] (div_short; the bounds here are one binade
+// inside, and binary16 ends at 65504).
+inline bool general_plain(const RunArgs &a, int prec)
+{
+    if (a.n_sets > 1) return true;
+    for (int j = 0; j < a.M; ++j) {
+        if (a.law[j] == 1 && prec >= MIXED_F16 && a.hill_a[j] != 0.0) {
+            const bool f16 = prec == MIXED_F16 || prec == UNIFORM_F16;
+            if (!(a.hill_a[j] >= 0x1p-29 && a.hill_a[j] <= (f16 ? 65504.0 : 0x1p30))) return true;
+        }
+        for (int i = 0; i < a.N; ++i) {
+            const bool read = a.law[j] == 1 ? a.hill_reg[j] == i : a.order[j][i] > 0 && !a.folded[j][i];
+            if (a.stoich[j][i] > 1024 || a.stoich[j][i] < -1024) return true;
+            if ((read || a.stoich[j][i] != 0) && a.x0[i] >= (1 << 23)) return true;
+        }
+    }
+    return false;
 }
 
 template <int PREC, int SR>
@@ -446,7 +466,7 @@ __device__ __forceinline__ void run_queue_general(const RunArgs &a, const typena
         if (__ballot_sync(0xFFFFFFFFu, L.active) == 0u) break;
 
         const int64_t room = a.max_events - L.n;
-        bool outside = room < 2 || L.n > max_fast || T.odd != 0;
+        bool outside = room < 2 || L.n > max_fast;
 #pragma unroll 1
         for (int i = 0; i < a.N; ++i)
             if ((T.moving >> i) & 1) outside = outside || L.x[i * L.bd] >= (1 << 23);
@@ -505,8 +525,8 @@ __device__ __forceinline__ void run_queue_general(const RunArgs &a, const typena
             for (int s = 0; s < slice && G.active; ++s) {
                 const uint64_t blk = (uint64_t)(G.n >> 1);
                 const uint4 u = philox4x32_10(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), G.traj, 0u), a.key0, a.key1);
-                if ((G.n & 1) == 0) ssa_step_general<PREC, SR>(a, G, u.x, u.y, smp, t_end);
-                if (G.active && (G.n & 1)) ssa_step_general<PREC, SR>(a, G, u.z, u.w, smp, t_end);
+                if ((G.n & 1) == 0) ssa_step_general<PREC, SR, false>(a, G, u.x, u.y, smp, t_end);
+                if (G.active && (G.n & 1)) ssa_step_general<PREC, SR, false>(a, G, u.z, u.w, smp, t_end);
             }
             L.t = G.t;
             L.n = G.n;

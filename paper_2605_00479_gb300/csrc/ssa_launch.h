@@ -101,28 +101,39 @@ inline int default_block(long long n, int sms, int p256, int p128)
     return block;
 }
 
+template <class ModelF, bool PLAIN>
+auto pick_kernel(int prec, int sr) -> void (*)(const RunArgs)
+{
+    switch (prec) {
+    case FP64: return ssa_kernel<ModelF, FP64, 0, PLAIN>;
+    case FP32: return ssa_kernel<ModelF, FP32, 0, PLAIN>;
+    case MIXED_F16: return sr ? ssa_kernel<ModelF, MIXED_F16, 1, PLAIN> : ssa_kernel<ModelF, MIXED_F16, 0, PLAIN>;
+    case MIXED_BF16: return sr ? ssa_kernel<ModelF, MIXED_BF16, 1, PLAIN> : ssa_kernel<ModelF, MIXED_BF16, 0, PLAIN>;
+    case UNIFORM_F16:
+        return sr == 2 ? ssa_kernel<ModelF, UNIFORM_F16, 2, PLAIN>
+                       : (sr ? ssa_kernel<ModelF, UNIFORM_F16, 1, PLAIN> : ssa_kernel<ModelF, UNIFORM_F16, 0, PLAIN>);
+    case UNIFORM_BF16:
+        return sr == 2 ? ssa_kernel<ModelF, UNIFORM_BF16, 2, PLAIN>
+                       : (sr ? ssa_kernel<ModelF, UNIFORM_BF16, 1, PLAIN> : ssa_kernel<ModelF, UNIFORM_BF16, 0, PLAIN>);
+    default: return nullptr;
+    }
+}
+
 // Shared launch logic: choose the kernel for (prec, sr), size the grid from
 // occupancy (persistent: enough lanes to fill the GPU, no more than the work).
 template <class ModelF>
 cudaError_t launch_family(const RunArgs &a, int prec, int sr, LaunchConfig cfg, cudaStream_t stream, int *grid_out)
 {
-    using K = void (*)(const RunArgs);
-    K k = nullptr;
-    switch (prec) {
-    case FP64: k = ssa_kernel<ModelF, FP64, 0>; break;
-    case FP32: k = ssa_kernel<ModelF, FP32, 0>; break;
-    case MIXED_F16: k = sr ? ssa_kernel<ModelF, MIXED_F16, 1> : ssa_kernel<ModelF, MIXED_F16, 0>; break;
-    case MIXED_BF16: k = sr ? ssa_kernel<ModelF, MIXED_BF16, 1> : ssa_kernel<ModelF, MIXED_BF16, 0>; break;
-    case UNIFORM_F16:
-        k = sr == 2 ? ssa_kernel<ModelF, UNIFORM_F16, 2>
-                    : (sr ? ssa_kernel<ModelF, UNIFORM_F16, 1> : ssa_kernel<ModelF, UNIFORM_F16, 0>);
-        break;
-    case UNIFORM_BF16:
-        k = sr == 2 ? ssa_kernel<ModelF, UNIFORM_BF16, 2>
-                    : (sr ? ssa_kernel<ModelF, UNIFORM_BF16, 1> : ssa_kernel<ModelF, UNIFORM_BF16, 0>);
-        break;
-    default: return cudaErrorInvalidValue;
+    constexpr bool kGeneral = std::is_same<ModelF, GeneralModel>::value;
+    bool lists = false;                      // the general kernel with lists and columns
+    void (*k)(const RunArgs) = nullptr;
+    if constexpr (kGeneral) {
+        lists = !general_plain(a, prec);
+        k = lists ? pick_kernel<ModelF, false>(prec, sr) : pick_kernel<ModelF, true>(prec, sr);
+    } else {
+        k = pick_kernel<ModelF, false>(prec, sr);
     }
+    if (!k) return cudaErrorInvalidValue;
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -132,9 +143,9 @@ cudaError_t launch_family(const RunArgs &a, int prec, int sr, LaunchConfig cfg, 
     // attribute gets the same value (the largest, 41 KB) on every call, so calls
     // from several threads do not lower it for each other.
     auto columns = [&](int b) -> size_t {
-        return std::is_same<ModelF, GeneralModel>::value && a.n_sets == 1 ? general_columns(a.N, a.M, prec, b) : 0;
+        return lists ? general_columns(a.N, a.M, prec, b) : 0;
     };
-    if (columns(256) > 0) {
+    if (lists) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)general_columns(kMaxN, kMaxM, prec, 256));
         if (e != cudaSuccess) return e;
@@ -146,7 +157,9 @@ cudaError_t launch_family(const RunArgs &a, int prec, int sr, LaunchConfig cfg, 
         if (e != cudaSuccess) return e;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p128, k, 128, columns(128));
         if (e != cudaSuccess) return e;
-        block = default_block(a.n_work, sms, p256, p128);
+        // binary64 without lists: large blocks, which pack best (64 sets x 8
+        // trajectories of a 16-reaction network: 64 threads 9.1 ms, 256 7.6)
+        block = kGeneral && !lists && prec == FP64 ? 256 : default_block(a.n_work, sms, p256, p128);
     }
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, columns(block));
     if (e != cudaSuccess) return e;
