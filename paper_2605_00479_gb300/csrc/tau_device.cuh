@@ -197,14 +197,20 @@ __device__ inline int64_t first_leap_after(double s, double tau)
 // per instruction (Schloegl, tau = 0.005).  So a leap runs in two phases:
 //   1. every channel gets one Philox block: four uniforms of the
 //      multiplication method, or the rejection method's first quick test.
-//      What that does not settle is marked pending (its state in shared
-//      memory);
+//      What that does not settle is marked pending (its product, or the
+//      candidate left for the slow test, in shared memory);
 //   2. every lane works through its own pending channels, one block or
 //      rejection round an iteration, so lanes wait only for the largest total
 //      of a lane, not for the largest of every channel.
-// Quantities that only the slow test reads are computed only there.  Measured (GB300, Schloegl fp32, 1.5 10^5 trajectories,
-// 2000 leaps): 51.1 -> 28.4 ms, 23.5 ms with the slow test decided by hardware
-// logarithms (Rejection::settle).
+// Quantities that only the slow test reads are computed only there.  Measured
+// (GB300, Schloegl fp32, 1.5 10^5 trajectories, 2000 leaps): 51.1 -> 28.4 ms, 23.4
+// ms with the slow test decided by hardware logarithms (Rejection::settle).  In
+// binary64 every operation costs 64 cycles a warp whatever its lanes, so there
+// comparisons and counts are integer, and the first round's candidate is kept
+// for the slow test (telegraph 1.97 -> 1.69 ms, Schloegl 2 10^4 240 -> 210 ms;
+// before the phases 1.87 and birth-death at lambda = 5000 7.3 against 7.4 now).
+// A network without a compiled structure adds its changes up species by species
+// in a register (16 reactions, fp32, 4 10^4 trajectories: 6.5 -> 5.3 ms).
 template <class R>
 struct SamplerMath;
 template <>
@@ -223,6 +229,10 @@ struct SamplerMath<float> {
         if (x < 0x1p22f) return __float_as_int(x + 0x1.8p23f) - 0x4B400000;
         return (int64_t)x;
     }
+    // a settled draw as its column holds it
+    static __device__ __forceinline__ float draw(int k) { return (float)k; }
+    static __device__ __forceinline__ float draw(float k) { return k; }
+    static __device__ __forceinline__ int64_t fired(float d) { return to_int(d); }
     static __device__ __forceinline__ float logfact(float k, const float *small) { return k < 10.0f ? small[(int)k] : logfact_f32(k); }
 };
 template <>
@@ -236,33 +246,47 @@ struct SamplerMath<double> {
     static __device__ __forceinline__ double down(double x) { return floor(x); }
     static __device__ __forceinline__ int64_t to_int(double x)
     {
-        if (x < 0x1p30) return __double2loint(x + 0x1.8p52);
+        if (later(0x1p30, x)) return __double2loint(x + 0x1.8p52);
         return (int64_t)x;
     }
+    // a settled draw as its column holds it: an integer, so that the
+    // multiplication method's takes no binary64 operation
+    static __device__ __forceinline__ double draw(int k) { return __longlong_as_double((long long)k); }
+    static __device__ __forceinline__ double draw(double k) { return __longlong_as_double(to_int(k)); }
+    static __device__ __forceinline__ int64_t fired(double d) { return __double_as_longlong(d); }
     static __device__ __forceinline__ double logfact(double k, const double *small) { return k < 10.0 ? small[(int)k] : logfact_f64(k); }
 };
 
-// The rejection method's constants of lambda that every round needs.
+// The rejection method's constants of lambda that every round needs.  Positive
+// values are compared by later(): in binary64 an integer comparison, where one
+// on the binary64 pipe costs 64 cycles a warp.
 template <class R>
 struct Rejection {
-    R slam, b, a, vr;
+    R slam, b, a;
     __device__ __forceinline__ explicit Rejection(R lam)
     {
         using Q = SamplerMath<R>;
         slam = Q::root(lam);
         b = R(sizeof(R) == 8 ? 0.931 : 0.931f) + R(sizeof(R) == 8 ? 2.53 : 2.53f) * slam;
         a = R(sizeof(R) == 8 ? -0.059 : -0.059f) + R(sizeof(R) == 8 ? 0.02483 : 0.02483f) * b;
-        vr = R(sizeof(R) == 8 ? 0.9277 : 0.9277f) - Q::div(R(sizeof(R) == 8 ? 3.6224 : 3.6224f), b - R(2));
+    }
+    // U of word w0, the distance us of |U| from 1/2 and V of word w1
+    __device__ __forceinline__ R point(uint32_t w0, uint32_t w1, R &us, R &V) const
+    {
+        using Q = SamplerMath<R>;
+        const R U = Q::half_open(w0) - R(0.5);
+        V = Q::positive(w1);
+        us = R(0.5) - (U < R(0) ? -U : U);
+        return U;
     }
     // One round on words (w0, w1): true when it settles without the slow
     // test; then kf is the draw, or -1 when the round is rejected.
     __device__ __forceinline__ bool quick(R lam, uint32_t w0, uint32_t w1, R &us, R &V, R &kf) const
     {
         using Q = SamplerMath<R>;
-        const R U = Q::half_open(w0) - R(0.5);
-        V = Q::positive(w1);
-        us = R(0.5) - (U < R(0) ? -U : U);
-        if (!(us > R(0))) {
+        const R vr = R(sizeof(R) == 8 ? 0.9277 : 0.9277f) - Q::div(R(sizeof(R) == 8 ? 3.6224 : 3.6224f), b - R(2));
+        const R U = point(w0, w1, us, V);
+        if (!later(us, R(0))) {
             kf = R(-1);
             return true;
         }
@@ -270,9 +294,9 @@ struct Rejection {
         v = v + lam;
         v = v + R(sizeof(R) == 8 ? 0.43 : 0.43f);
         kf = Q::down(v);
-        if (us >= R(sizeof(R) == 8 ? 0.07 : 0.07f) && V <= vr) return true;
+        if (!later(R(sizeof(R) == 8 ? 0.07 : 0.07f), us) && !later(V, vr)) return true;   // vr >= 0.4 from lambda = 10 on
         const R kmax = lam + R(64) * slam + R(64);
-        if (kf < R(0) || (us < R(sizeof(R) == 8 ? 0.013 : 0.013f) && V > us) || kf > kmax) {
+        if (kf < R(0) || (later(R(sizeof(R) == 8 ? 0.013 : 0.013f), us) && later(V, us)) || later(kf, kmax)) {
             kf = R(-1);
             return true;
         }
@@ -321,19 +345,23 @@ struct Rejection {
     }
 };
 
+// (binary32 counts in binary32: 1% faster than in integers)
+template <class R>
+using CountOf = typename std::conditional<sizeof(R) == 8, int, R>::type;
+
 // Four uniforms of the multiplication method: p *= v; counts the products
 // above L.  True when the last one is not (the draw is settled).
 template <class R>
-__device__ __forceinline__ bool multiply_block(R &p, R L, uint4 u, R &count)
+__device__ __forceinline__ bool multiply_block(R &p, R L, uint4 u, CountOf<R> &count)
 {
     using Q = SamplerMath<R>;
-    R c = R(0);
-    p = p * Q::positive(u.x); if (p > L) c = c + R(1);
-    p = p * Q::positive(u.y); if (p > L) c = c + R(1);
-    p = p * Q::positive(u.z); if (p > L) c = c + R(1);
-    p = p * Q::positive(u.w); if (p > L) c = c + R(1);
+    CountOf<R> c = 0;
+    p = p * Q::positive(u.x); if (later(p, L)) c += 1;
+    p = p * Q::positive(u.y); if (later(p, L)) c += 1;
+    p = p * Q::positive(u.z); if (later(p, L)) c += 1;
+    p = p * Q::positive(u.w); if (later(p, L)) c += 1;
     count = c;
-    return !(p > L);
+    return !later(p, L);
 }
 
 // f(j) for every channel: unrolled for compiled structures (j a constant),
@@ -385,13 +413,18 @@ __device__ __forceinline__ void tau_leap(const RunArgs &a, Lane<Model, PREC> &L,
         if constexpr (kGeneral) general_propensities<PREC, SR>(a, L, R, prop);
         else static_propensities<Model, PREC, SR>(a, L, R, prop);
         tau_channels<Model>(a, [&](int j) {
-
             P v;
             if constexpr (Tr::kF64) v = prop[j] * a.tau;
             else if constexpr (Tr::kUniform) v = R.rnd(prop[j] * tau16, lam_op + j);
             else v = prop[j] * tau32;
-            if (v != v) bad |= ST_NAN;
-            else if (v == P(__int_as_float(0x7F800000))) bad |= ST_OVERFLOW;
+            if constexpr (Tr::kF64) {
+                const uint64_t b = (uint64_t)__double_as_longlong(v), inf = 0x7FF0000000000000ull;
+                if ((b & 0x7FFFFFFFFFFFFFFFull) > inf) bad |= ST_NAN;
+                else if (b == inf) bad |= ST_OVERFLOW;
+            } else {
+                if (v != v) bad |= ST_NAN;
+                else if (v == P(__int_as_float(0x7F800000))) bad |= ST_OVERFLOW;
+            }
             col[j * bd] = v;
         });
     }
@@ -411,28 +444,38 @@ __device__ __forceinline__ void tau_leap(const RunArgs &a, Lane<Model, PREC> &L,
         // phase 1: one block a channel
         uint32_t pend = 0u;
         tau_channels<Model>(a, [&](int j) {
-
             const P lam = col[j * bd];
-            P k = P(0);
-            if (lam > P(0)) {
+            P d = Q::draw(0);
+            if (later(lam, P(0))) {
                 const uint4 u = ph.block(0u, 2u + (uint32_t)j, a.key0, a.key1);
-                if (lam < P(10)) {
+                if (later(P(10), lam)) {
                     const P e = Q::exp(-lam);
                     P p = P(1);
-                    if (!multiply_block<P>(p, e, u, k)) {
+                    CountOf<P> c;
+                    if (multiply_block<P>(p, e, u, c)) {
+                        d = Q::draw(c);
+                    } else {
                         pend |= 1u << j;
                         colL[j * bd] = e;
-                        k = p;
+                        d = p;
                     }
                 } else {
                     const Rejection<P> rej(lam);
-                    P us, V;
-                    if (!rej.quick(lam, u.x, u.y, us, V, k) || k < P(0)) pend |= 1u << j;
+                    P us, V, k;
+                    if (rej.quick(lam, u.x, u.y, us, V, k) && !later(P(0), k)) {
+                        d = Q::draw(k);
+                    } else {   // k: the first round's candidate for the slow test, or -1
+                        pend |= 1u << j;
+                        d = k;
+                    }
                 }
             }
-            colK[j * bd] = k;
+            colK[j * bd] = d;
         });
-        // phase 2: the lane's pending channels
+        // phase 2: the lane's pending channels.  The first round's candidate is kept
+        // in binary64 only; in binary32 another round is cheaper than the branch
+        // (Schloegl, 1.5 10^5 trajectories: 23.4 against 23.8 ms).
+        constexpr bool kKeep = Tr::kF64;
         int j = 0, it = 0;
         P lam = P(0), e = P(0), p = P(0);
         auto take = [&]() {
@@ -440,69 +483,50 @@ __device__ __forceinline__ void tau_leap(const RunArgs &a, Lane<Model, PREC> &L,
             lam = col[j * bd];
             e = colL[j * bd];
             p = colK[j * bd];
-            it = lam < P(10) ? 1 : 0;
+            it = later(P(10), lam) || (kKeep && later(P(0), p)) ? 1 : 0;
         };
         if (pend) take();
         while (pend) {
-            const bool product = lam < P(10);
+            const bool product = later(P(10), lam);
             const uint4 u = ph.block(product ? (uint32_t)it : (uint32_t)(it >> 1), 2u + (uint32_t)j, a.key0, a.key1);
             bool done;
-            P k;
+            P d;
             if (product) {
-                P c;
+                CountOf<P> c;
                 done = multiply_block<P>(p, e, u, c);
-                k = P(4 * it) + c;
+                c += 4 * it;
                 if (it == 249 && !done) {   // 1000 uniforms: the bound of the method
                     done = true;
-                    k = P(999);
+                    c = 999;
                 }
+                d = Q::draw(c);
             } else {
                 const Rejection<P> rej(lam);
-                P us, V;
+                P us, V, k = p;
                 const bool second = (it & 1) != 0;
-                done = rej.quick(lam, second ? u.z : u.x, second ? u.w : u.y, us, V, k);
-                if (done) done = k >= P(0);
+                const uint32_t w0 = second ? u.z : u.x, w1 = second ? u.w : u.y;
+                bool settled = false;
+                if (kKeep && it == 0) rej.point(w0, w1, us, V);   // its candidate is k
+                else settled = rej.quick(lam, w0, w1, us, V, k);
+                if (settled) done = !later(P(0), k);
                 else done = rej.slow(lam, us, V, k, small);
                 if (it == 99 && !done) {    // 100 rounds
                     done = true;
                     k = Q::down(lam);
                 }
+                d = Q::draw(k);
             }
             it += 1;
             if (done) {
-                colK[j * bd] = k;
+                colK[j * bd] = d;
                 pend &= pend - 1u;
                 if (pend) take();
             }
         }
         // x += sum_j nu_j k_j
-        int64_t dx[Model::N];
-#pragma unroll
-        for (int i = 0; i < Model::N; ++i) dx[i] = 0;
         int64_t fired = 0;
-        if constexpr (kGeneral) {
-#pragma unroll 1
-            for (int c = 0; c < a.M; ++c) {
-                const int64_t k = Q::to_int(colK[c * bd]);
-                fired += k;
-#pragma unroll 1
-                for (int i = 0; i < a.N; ++i) dx[i] += k * (int64_t)a.stoich[c][i];
-            }
-        } else {
-            unroll<Model::M>([&](auto J) {
-                constexpr int c = decltype(J)::value;
-                const int64_t k = Q::to_int(colK[c * bd]);
-                fired += k;
-                unroll<Model::N>([&](auto I) {
-                    constexpr int i = decltype(I)::value;
-                    const int nu = Model::template nu<c, i>(a);
-                    if (nu != 0) dx[i] += k * (int64_t)nu;
-                });
-            });
-        }
-        L.ev += fired;
-        auto move = [&](int i) {
-            int64_t v = (int64_t)L.x[i] + dx[i];
+        auto move = [&](int i, int64_t dx) {
+            int64_t v = (int64_t)L.x[i] + dx;
             if (v < 0) {
                 v = 0;
                 L.status |= ST_TAU_CLAMPED;
@@ -511,11 +535,48 @@ __device__ __forceinline__ void tau_leap(const RunArgs &a, Lane<Model, PREC> &L,
             L.x[i] = (int)v;
         };
         if constexpr (kGeneral) {
+            // one species after the other, so that its sum stays in a register;
+            // in binary32 from draws narrowed to 32 bits where all of them fit
+            int32_t *const narrow = reinterpret_cast<int32_t *>(col);   // lambda is no longer needed
+            bool wide = Tr::kF64;
 #pragma unroll 1
-            for (int i = 0; i < a.N; ++i) move(i);
+            for (int c = 0; c < M; ++c) {
+                const int64_t k = Q::fired(colK[c * bd]);
+                fired += k;
+                if constexpr (!Tr::kF64) {
+                    narrow[c * bd] = (int32_t)k;
+                    wide = wide || k != (int64_t)(int32_t)k;
+                }
+            }
+#pragma unroll 1
+            for (int i = 0; i < a.N; ++i) {
+                int64_t dx = 0;
+                if (wide) {
+#pragma unroll 4
+                    for (int c = 0; c < M; ++c) dx += Q::fired(colK[c * bd]) * (int64_t)a.stoich[c][i];
+                } else {
+#pragma unroll 4
+                    for (int c = 0; c < M; ++c) dx += (int64_t)narrow[c * bd] * (int64_t)a.stoich[c][i];
+                }
+                move(i, dx);
+            }
         } else {
-            unroll<Model::N>([&](auto I) { move(decltype(I)::value); });
+            int64_t dx[Model::N];
+#pragma unroll
+            for (int i = 0; i < Model::N; ++i) dx[i] = 0;
+            unroll<Model::M>([&](auto J) {
+                constexpr int c = decltype(J)::value;
+                const int64_t k = Q::fired(colK[c * bd]);
+                fired += k;
+                unroll<Model::N>([&](auto I) {
+                    constexpr int i = decltype(I)::value;
+                    const int nu = Model::template nu<c, i>(a);
+                    if (nu != 0) dx[i] += k * (int64_t)nu;
+                });
+            });
+            unroll<Model::N>([&](auto I) { move(decltype(I)::value, dx[decltype(I)::value]); });
         }
+        L.ev += fired;
         L.n += 1;
         if (L.n >= a.n_leaps) tau_finish<Model, PREC>(a, L);
     }
