@@ -413,7 +413,9 @@ cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t s)
     size_t smem = (size_t)a.stages * stage + 128;
     const size_t floor_bytes = per_sm / (cap_ctas + 1) + 1 - reserve;
     if (smem < floor_bytes) smem = floor_bytes;
-    cudaError_t e = cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // always the same value (what is left beside the kernel's static words), so
+    // calls from several threads do not lower it for each other
+    cudaError_t e = cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_dyn - 64);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)tiles, (unsigned)(g.N / a.ntile));
     gemm_kernel<<<grid, 128, smem, s>>>(a);

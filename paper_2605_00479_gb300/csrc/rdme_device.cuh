@@ -1204,7 +1204,9 @@ cudaError_t rdme_launch_mode(const RdmeArgs &A, int max_block, int blocks_per_sm
     const int block = rdme_block_size_for(A, (int)sizeof(P), kEpochs, max_block, smem_limit);
     if (block < 32) return cudaErrorInvalidConfiguration;
     const size_t bytes = rdme_layout(A.a.K, A.S, A.T, A.n_stored, block, (int)sizeof(P), kEpochs).total;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    // the device's limit on every call, so that lattices of other sizes, launched
+    // by other threads, do not lower it
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     e = cudaGetDevice(&dev);
