@@ -254,9 +254,10 @@ int ssa_tau_run(const ssa_model *model, int64_t n_traj, uint64_t traj_offset, co
  *   max_events    events (reactions + hops) per trajectory, 0..2^32-2
  *   out           device [K][S][N][n_traj], trajectory index fastest
  *   other arguments as ssa_ensemble_run (n_events counts reactions and hops)
- * Allocates a work-queue counter, the [S][N] initial-state table and a table
- * of voxel sums (128 KiB, 256 KiB in fp64) with stream-ordered allocation and
- * frees them after the launch.
+ * Allocates a work-queue counter, the [S][N] initial-state table and, for
+ * birth-death and Schloegl structures without stochastic rounding, a table of
+ * voxel sums (128 KiB, 256 KiB in fp64) with stream-ordered allocation and frees
+ * them after the launch.
  * Errors: SSA_EINVAL (arguments; lattice too large), SSA_ENOMEM, SSA_ECUDA.
  */
 int ssa_rdme_run(const ssa_model *model, int nx, int ny, int nz, const double *diffusion, int64_t n_traj,

@@ -56,8 +56,9 @@ struct RdmeArgs {
 // (M <= 6), again S_M at [6], the value of one hop channel at [7] -- for counts
 // below kTableRows, filled by the voxel's own arithmetic before the launch and
 // read through the L1 cache.  A voxel is then one load instead of its chains:
-// three of them per event (two where no hop happens).  32-voxel Schloegl chain, 65536 lattices, mixed f16: 53.8 -> 48.6 ms; 17 voxels, 10^4 lattices,
-// fp64: 28.5 -> 20.6 ms.
+// three of them per event (two where no hop happens).  32-voxel Schloegl chain,
+// 65536 lattices, mixed f16: 53.8 -> 48.6 ms; 17 voxels, 10^4 lattices, fp64:
+// 28.5 -> 20.6 ms.
 constexpr int kTableRows = 4096;
 template <class Model, int SR>
 struct VoxelTable {
@@ -115,6 +116,14 @@ template <class Sx, bool NORM, int SR>
 struct VoxelTable<StaticModel<Sx, NORM>, SR> {
     static constexpr bool use = SR == 0 && RdmeSpecies<StaticModel<Sx, NORM>>::count() == 1 && Sx::M <= 6;
 };
+
+// Bytes of the table of a run, 0 where its kernel reads none: the same rule by
+// structure family (birth-death and Schloegl move one species), precision and rounding.
+inline size_t rdme_table_bytes(int family, int prec, int sr)
+{
+    const bool one = family == 1 || family == 2;
+    return one && !(sr && prec >= MIXED_F16) ? (size_t)kTableRows * 8 * (prec == FP64 ? 8 : 4) : 0;
+}
 
 // Stochastic-rounding words keyed by (op / 8, epoch, trajectory, tag).
 struct TagBits {
@@ -203,7 +212,7 @@ __device__ __forceinline__ int rdme_neighbour(const RdmeArgs &A, int v, int dir)
     }
 }
 
-// Partial sums over a voxel's channels with selection (shared by both paths).
+// General model: partial sums over a voxel's channels with selection.
 template <int PREC, int SR>
 struct ChannelSum {
     using Tr = ModeTraits<PREC>;
@@ -328,7 +337,6 @@ struct VoxelCounts {
 template <class Model, int PREC, int SR>
 struct VoxelModel {
     FastLane<Model, PREC, SR> L;
-    bool odd;
 };
 
 template <int PREC, int SR>
@@ -407,7 +415,7 @@ __device__ __forceinline__ typename ModeTraits<PREC>::P rdme_voxel_fast(const Rd
     unroll<N>([&](auto I) { X.x[decltype(I)::value] = rdme_get<Model, decltype(I)::value>(W, v); });
     P prop[M];
     uint16_t p16[M];
-    fast_propensities<true>(C.L, X, bits, prop, p16, C.odd);
+    fast_propensities<true>(C.L, X, bits, prop, p16, C.L.odd);
     const int nnb = __popc((unsigned)W.nbmask[v]);
     P hv[N];
     int op = ChainPlan<Model>::first_slot(M);
@@ -624,44 +632,21 @@ __device__ void rdme_init(const RdmeArgs &A, const RdmeView<PREC> &W, const Voxe
     L.active = true;
 }
 
-// Apply channel c of voxel v; returns the hop's destination voxel or -1.
-template <class Model, int PREC>
+// General model.  Apply channel c of voxel v; returns the hop's destination
+// voxel or -1.
+template <int PREC>
 __device__ __forceinline__ int rdme_apply(const RdmeArgs &A, const RdmeView<PREC> &W, int v, int c, bool &negative)
 {
     const RunArgs &a = A.a;
     negative = false;
     if (c < a.M) {
-        if constexpr (RdmeSpecies<Model>::kStatic) {
-            unroll<Model::N>([&](auto I) {      // branch-free: d_i = nu[c][i] by selects
-                constexpr int i = decltype(I)::value;
-                constexpr int s = RdmeSpecies<Model>::slot(i);
-                if constexpr (s >= 0) {
-                    int d = 0;
-                    bool moves = false;
-                    unroll<Model::M>([&](auto J) {
-                        constexpr int j = decltype(J)::value;
-                        const int nu = Model::template nu<j, i>(a);
-                        if (nu != 0) {
-                            d = (c == j) ? nu : d;
-                            moves = true;
-                        }
-                    });
-                    if (moves) {
-                        int &xr = W.at(v, s);
-                        xr += d;
-                        negative = negative || (xr < 0);
-                    }
-                }
-            });
-        } else {
 #pragma unroll 1
-            for (int i = 0; i < a.N; ++i) {
-                const int d = a.stoich[c][i];
-                if (d == 0) continue;
-                int &xr = W.at(v, i);
-                xr += d;
-                negative = negative || (xr < 0);
-            }
+        for (int i = 0; i < a.N; ++i) {
+            const int d = a.stoich[c][i];
+            if (d == 0) continue;
+            int &xr = W.at(v, i);
+            xr += d;
+            negative = negative || (xr < 0);
         }
         return -1;
     }
@@ -684,23 +669,9 @@ __device__ __forceinline__ int rdme_apply(const RdmeArgs &A, const RdmeView<PREC
         }
     }
     const int w = rdme_neighbour(A, v, dir);
-    if constexpr (RdmeSpecies<Model>::kStatic) {
-        unroll<Model::N>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            constexpr int s = RdmeSpecies<Model>::slot(i);
-            if constexpr (s >= 0) {
-                if (i == species) {
-                    W.at(v, s) -= 1;
-                    W.at(w, s) += 1;
-                    negative = W.at(v, s) < 0;
-                }
-            }
-        });
-    } else {
-        W.at(v, species) -= 1;
-        W.at(w, species) += 1;
-        negative = W.at(v, species) < 0;
-    }
+    W.at(v, species) -= 1;
+    W.at(w, species) += 1;
+    negative = W.at(v, species) < 0;
     return w;
 }
 
@@ -820,7 +791,7 @@ __device__ __forceinline__ void rdme_event(const RdmeArgs &A, const RdmeView<PRE
         return;
     }
     bool negative = false;
-    const int w = rdme_apply<Model, PREC>(A, W, v, c, negative);
+    const int w = rdme_apply<PREC>(A, W, v, c, negative);
     L.t = t_new;
     L.n += 1;
     if (negative) {
@@ -880,20 +851,14 @@ __device__ __forceinline__ void rdme_event(const RdmeArgs &A, const RdmeView<PRE
     }
 }
 
-// One event, compiled structures.  What bounds it is instruction count (the
-// columns are conflict-free shared memory): the arithmetic is that of
-// ssa_fast.cuh, a changed leaf climbs the tree with one addition a level (a
-// node is the sum of two, in either order), and a hop's destination climbs
-// first, so both paths' common part ends with the final values.  Measured
-// (GB300, 32-voxel Schloegl chain, mixed f16, 65536 lattices): 64.1 -> 53.8 ms;
-// mixed f16 SR 59.7 -> 46.6 ms (to t = 0.1).  E: -log u1; w1: the second word.
-template <class Model, int PREC>
+// Destination of the idx-th hop channel out of voxel v (neighbours: mask nb).
 __device__ __forceinline__ int rdme_hop_target(const RdmeArgs &A, unsigned nb, int v, int idx)
 {
     for (int q = 0; q < idx; ++q) nb &= nb - 1u;
     return rdme_neighbour(A, v, __ffs((int)nb) - 1);
 }
 
+// A changed leaf's value up to the root, which is returned.
 template <int PREC, int SR>
 __device__ __forceinline__ typename ModeTraits<PREC>::P rdme_climb(const RdmeArgs &A, const RdmeView<PREC> &W, int leaf,
                                                                    typename ModeTraits<PREC>::P val, uint32_t e, uint32_t traj)
@@ -914,6 +879,13 @@ __device__ __forceinline__ typename ModeTraits<PREC>::P rdme_climb(const RdmeArg
     return val;
 }
 
+// One event, compiled structures.  What bounds it is instruction count (the
+// columns are conflict-free shared memory): the arithmetic is that of
+// ssa_fast.cuh, a changed leaf climbs the tree with one addition a level (a
+// node is the sum of two, in either order), and a hop's destination climbs
+// first, so both paths' common part ends with the final values.  Measured
+// (GB300, 32-voxel Schloegl chain, mixed f16, 65536 lattices): 64.1 -> 53.8 ms;
+// mixed f16 SR 59.7 -> 46.6 ms (to t = 0.1).  E: -log u1; w1: the second word.
 template <class Model, int PREC, int SR>
 __device__ __forceinline__ void rdme_event_fast(const RdmeArgs &A, const RdmeView<PREC> &W,
                                                 const VoxelModel<Model, PREC, SR> &C, RLane<PREC> &L,
@@ -1041,7 +1013,7 @@ __device__ __forceinline__ void rdme_event_fast(const RdmeArgs &A, const RdmeVie
             if constexpr (s >= 0) {
                 if ((W.dmask >> i) & 1u) {
                     if (idx >= 0 && idx < nnb) {
-                        w = rdme_hop_target<Model, PREC>(A, nb, v, idx);
+                        w = rdme_hop_target(A, nb, v, idx);
                         W.at(v, s) -= 1;
                         W.at(w, s) += 1;
                         negative = W.at(v, s) < 0;
@@ -1134,7 +1106,6 @@ __global__ void __launch_bounds__(256) rdme_kernel(const __grid_constant__ RdmeA
     VoxelModel<Model, PREC, SR> C;
     if constexpr (RdmeSpecies<Model>::kStatic) {
         fast_init(a, C.L, 0);      // the constants; a lattice has one parameter set
-        C.odd = C.L.odd;
     }
     bool drained = false;
     for (;;) {
@@ -1224,6 +1195,7 @@ cudaError_t rdme_launch_mode(const RdmeArgs &A, int max_block, int blocks_per_sm
     *grid_out = (int)grid;
     *block_out = block;
     if constexpr (VoxelTable<Model, SR>::use) {
+        if (!A.table) return cudaErrorInvalidValue;
         rdme_table_kernel<Model, PREC><<<kTableRows / 128, 128, 0, stream>>>(A);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -817,7 +817,7 @@ int ssa_rdme_run(const ssa_model *model, int nx, int ny, int nz, const double *d
     const size_t lat_bytes = sizeof(int32_t) * (size_t)S * (size_t)N;
     char *d = nullptr;
     const size_t table_at = align_up(256 + lat_bytes, 256);   // VoxelTable rows of the kernels that read them
-    const size_t table_bytes = (size_t)ssa::kTableRows * 8 * (size_t)elem;
+    const size_t table_bytes = ssa::rdme_table_bytes(model->family, precision, rounding);
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&d), table_at + table_bytes, s);
     if (e != cudaSuccess) {
         delete A;
@@ -826,7 +826,7 @@ int ssa_rdme_run(const ssa_model *model, int nx, int ny, int nz, const double *d
     }
     A->a.queue_head = reinterpret_cast<unsigned long long *>(d);
     A->x0_lat = reinterpret_cast<const int32_t *>(d + 256);
-    A->table = d + table_at;
+    A->table = table_bytes ? d + table_at : nullptr;
     e = cudaMemsetAsync(d, 0, sizeof(unsigned long long), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d + 256, x0, lat_bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) {
