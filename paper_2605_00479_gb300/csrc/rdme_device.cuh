@@ -851,27 +851,32 @@ __device__ __forceinline__ void rdme_event(const RdmeArgs &A, const RdmeView<PRE
     }
 }
 
-// Destination of the idx-th hop channel out of voxel v (neighbours: mask nb).
+// Destination of the idx-th hop channel out of voxel v (neighbours: mask nb), by
+// selects: lanes hop in different directions.
 __device__ __forceinline__ int rdme_hop_target(const RdmeArgs &A, unsigned nb, int v, int idx)
 {
-    for (int q = 0; q < idx; ++q) nb &= nb - 1u;
-    return rdme_neighbour(A, v, __ffs((int)nb) - 1);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) nb &= idx > q ? nb - 1u : nb;
+    const int dir = __ffs((int)nb) - 1;
+    const int stride = dir < 2 ? 1 : (dir < 4 ? A.nx : A.nx * A.ny);
+    return (dir & 1) ? v + stride : v - stride;
 }
 
-// A changed leaf's value up to the root, which is returned.
+// A changed leaf's value `levels` up the tree; returns the last node's.
 template <int PREC, int SR>
 __device__ __forceinline__ typename ModeTraits<PREC>::P rdme_climb(const RdmeArgs &A, const RdmeView<PREC> &W, int leaf,
-                                                                   typename ModeTraits<PREC>::P val, uint32_t e, uint32_t traj)
+                                                                   typename ModeTraits<PREC>::P val, uint32_t e, uint32_t traj,
+                                                                   int levels)
 {
     using P = typename ModeTraits<PREC>::P;
     int q = leaf;
     W.Node(q) = val;
-    P sib = A.depth > 0 ? W.Node(q ^ 1) : P(0);
+    P sib = levels > 0 ? W.Node(q ^ 1) : P(0);
 #pragma unroll 1
-    for (int l = 0; l < A.depth; ++l) {
+    for (int l = 0; l < levels; ++l) {
         const int up = q >> 1;
         const P s = sib;
-        if (l + 1 < A.depth) sib = W.Node(up ^ 1);   // the next level's, ahead of this level's store
+        if (l + 1 < levels) sib = W.Node(up ^ 1);   // the next level's, ahead of this level's store
         val = rdme_sum<PREC, SR>(A, val, s, up, e, traj);
         W.Node(up) = val;
         q = up;
@@ -883,9 +888,8 @@ __device__ __forceinline__ typename ModeTraits<PREC>::P rdme_climb(const RdmeArg
 // columns are conflict-free shared memory): the arithmetic is that of
 // ssa_fast.cuh, a changed leaf climbs the tree with one addition a level (a
 // node is the sum of two, in either order), and a hop's destination climbs
-// first, so both paths' common part ends with the final values.  Measured
-// (GB300, 32-voxel Schloegl chain, mixed f16, 65536 lattices): 64.1 -> 53.8 ms;
-// mixed f16 SR 59.7 -> 46.6 ms (to t = 0.1).  E: -log u1; w1: the second word.
+// first, up to where the paths meet.  Measured (GB300, 32-voxel Schloegl chain,
+// mixed f16, 65536 lattices): 64.1 -> 40.2 ms.  E: -log u1; w1: the second word.
 template <class Model, int PREC, int SR>
 __device__ __forceinline__ void rdme_event_fast(const RdmeArgs &A, const RdmeView<PREC> &W,
                                                 const VoxelModel<Model, PREC, SR> &C, RLane<PREC> &L,
@@ -1006,22 +1010,33 @@ __device__ __forceinline__ void rdme_event_fast(const RdmeArgs &A, const RdmeVie
             }
         });
     } else {
-        int idx = c - M;
-        unroll<N>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            constexpr int s = RdmeSpecies<Model>::slot(i);
-            if constexpr (s >= 0) {
-                if ((W.dmask >> i) & 1u) {
-                    if (idx >= 0 && idx < nnb) {
-                        w = rdme_hop_target(A, nb, v, idx);
-                        W.at(v, s) -= 1;
-                        W.at(w, s) += 1;
-                        negative = W.at(v, s) < 0;
+        // the hopping species' column by selects and one destination for all of them
+        // (destinations species by species made lanes wait for each other: lattices
+        // of the repressilator with six hopping species, 3 x 3 voxels, were slower
+        // than with the general event, fp32 7.34 -> 7.69 ms, mixed bf16 SR 11.8 ->
+        // 12.4; with this, rdme_hop_target's selects and the shorter climb 6.72 and 10.5)
+        int idx = c - M, col = 0;
+        if constexpr (RdmeSpecies<Model>::count() > 1) {
+            int dir = 0;
+            unroll<N>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                constexpr int s = RdmeSpecies<Model>::slot(i);
+                if constexpr (s >= 0) {
+                    if ((W.dmask >> i) & 1u) {
+                        const bool here = (unsigned)idx < (unsigned)nnb;
+                        col = here ? s : col;
+                        dir = here ? idx : dir;
+                        idx -= nnb;
                     }
-                    idx -= nnb;
                 }
-            }
-        });
+            });
+            idx = dir;
+        }
+        w = rdme_hop_target(A, nb, v, idx);
+        const int x = W.at(v, col) - 1;
+        W.at(v, col) = x;
+        W.at(w, col) += 1;
+        negative = x < 0;
     }
     L.t = t_new;
     L.n += 1;
@@ -1031,12 +1046,23 @@ __device__ __forceinline__ void rdme_event_fast(const RdmeArgs &A, const RdmeVie
         return;
     }
     const uint32_t e = (uint32_t)L.n;
-    if (w >= 0) {
-        if (W.epoch) W.epoch[w * W.bd] = e;
-        rdme_climb<PREC, SR>(A, W, T + w, rdme_voxel_fast<false>(A, W, C, w, e, L.traj, P(0), nullptr), e, L.traj);
+    auto renew = [&](int u, int levels) {
+        if (W.epoch) W.epoch[u * W.bd] = e;
+        return rdme_climb<PREC, SR>(A, W, T + u, rdme_voxel_fast<false>(A, W, C, u, e, L.traj, P(0), nullptr), e, L.traj,
+                                    levels);
+    };
+    // a hop's destination first, and only below the paths' common part: the other
+    // climb forms the rest.  Both in one copy of the voxel's code where several
+    // species move (dimer fp32, 3 x 3 voxels: 9.7 against 8.7 ms), in two for one
+    // species (Schloegl 4.35 against 4.07 ms).
+    const int below = w >= 0 ? 31 - __clz(v ^ w) : 0;
+    if constexpr (RdmeSpecies<Model>::count() == 1) {
+        if (w >= 0) renew(w, below);
+        L.a0 = renew(v, A.depth);
+    } else {
+#pragma unroll 1
+        for (int h = w >= 0 ? 0 : 1; h < 2; ++h) L.a0 = renew(h ? v : w, h ? A.depth : below);
     }
-    if (W.epoch) W.epoch[v * W.bd] = e;
-    L.a0 = rdme_climb<PREC, SR>(A, W, T + v, rdme_voxel_fast<false>(A, W, C, v, e, L.traj, P(0), nullptr), e, L.traj);
 }
 
 // Persistent RDME kernel: lanes refill from the work queue; each loop
