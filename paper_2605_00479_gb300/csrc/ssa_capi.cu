@@ -76,12 +76,16 @@ int g_longest_first = 1;
 int64_t g_park_events = 0;
 constexpr double kLongestFirstMinEvents = 4096.0;   // estimated events per trajectory
 // trajectories per multiprocessor: batches and fp64, single runs of the other
-// modes.  Schloegl, unsplit -> split, ms: mixed bf16 8 10^4 28.9 -> 30.1, 10^5
-// 32.2 -> 25.3, 2 10^5 38.0 -> 34.6, 3 10^5 52.6 -> 45.6; uniform f16 SR 1.5 10^5
-// 83.6 -> 74.3; uniform f16 RN 10^5 83.3 -> 62.0; repressilator 10^5 and below
-// unchanged.  fp64 6 10^4 420 -> 662: a warp of long trajectories holds its
-// scheduler's binary64 unit.  A sweep of three models x 500 sets x 64
-// trajectories 158 -> 238.
+// modes.  Unsplit -> split with the paired step, ms (mean of three seeds):
+//                              8 10^4          92416 (608)    1.2 10^5       1.5 10^5
+//   Schloegl mixed bf16        27.6 -> 28.1    30.2 -> 27.9   30.9 -> 32.0   33.9 -> 32.9
+//   Schloegl mixed f16 SR                      52.0 -> 53.0   55.8 -> 54.4   62.6 -> 55.6
+//   Schloegl uniform f16       71.5 -> 71.1    74.9 -> 74.7   84.2 -> 83.1   85.5 -> 83.7
+//   Schloegl uniform f16 SR    68.1 -> 70.9    69.6 -> 70.4   74.2 -> 73.0   82.7 -> 74.0
+//   repressilator mixed f16    29.6 -> 29.5    34.7 -> 34.0   43.5 -> 42.2   54.2 -> 52.7
+// (8 10^4: one seed); 3 10^5: mixed bf16 52.1 -> 45.8, uniform f16 126.9 -> 116.6.  fp64
+// 6 10^4 407 -> 663: a warp of long trajectories holds its scheduler's binary64
+// unit.  A sweep of three models x 500 sets x 64 trajectories 158 -> 238.
 constexpr int64_t kLongestFirstMinPerSM = 2048;
 constexpr int64_t kLongestFirstMinPerSM32 = 608;
 constexpr double kLongestFirstMinSpread = 4.0;      // batches: largest / smallest estimate over the sets

@@ -57,19 +57,21 @@ constexpr int kMaxK = 1024;
 #endif
 
 // Per kernel: a register budget, as 256-thread blocks per SM, where it was
-// measured to pay.  The one-species birth-death structure's round-to-nearest
-// kernels (not fp64) fit 64 registers: four blocks, 9.6 ms for 10^6
-// trajectories with 101 snapshots (mixed f16) against 10.2 ms at five blocks
-// (48 registers) and 10.0 ms at three.  Everywhere else every budget was slower
-// than the compiler's choice (three / four / five blocks: Schloegl mixed bf16
-// +4 / +6 / +4%, uniform f16 SR +6 / +21 / +27%, telegraph +6 / +5 / +6%,
-// repressilator +4 / +11 / +23%).
-
-//
-// General networks: three blocks (80 registers) except in fp64 and uniform SR.
-// 10^5 trajectories of a six-reaction network, fp32: 36.6 ms without a budget,
-// 23.8 / 24.6 ms at three / four blocks; repressilator with h = 3, mixed f16,
-// 51.9, 40.9 / 41.5; uniform f16 SR (10^4) 34.7, 38.9 / 41.4; fp64 7.5, 7.9 / 7.9.
+// measured to pay with the paired step.  Whole calls, ms, without a budget / at
+// three / four / five blocks:
+//   birth-death mixed f16, 10^6, 101 snapshots   7.81 /  7.26 /  7.10 /  7.44
+//   Schloegl mixed bf16, 10^6                   134.4 / 141.6 / 142.4 / 149.5
+//   Schloegl uniform f16 SR, 1.5 10^5            74.9 / 105.9 / 136.5 / 146.9
+//   Schloegl fp64, 2 10^4                       199.4 / 205.3 / 216.8 / 210.0
+//   telegraph mixed f16, 3 10^5                  2.37 /  2.18 /  2.41 /  2.63
+//   repressilator mixed f16, 5 10^4              23.7 /  24.2 /  27.1 /  28.9
+//   six-reaction general network fp32, 10^5      36.5 /  23.8 /  23.8 /  28.4
+//   repressilator with h = 3, mixed f16, 10^5    48.6 /  37.4 /  37.5 /  44.2
+//     the same, uniform f16 SR, 10^4             70.3 /  78.8 /  85.9 /  99.2
+//   six-reaction general network fp64, 10^4      36.9 /  37.3 /  39.3 /  42.1
+// So four blocks (64 registers) for the one-species round-to-nearest kernels
+// (not fp64), three (80) for general networks except in fp64 and uniform SR, the
+// compiler's choice elsewhere.
 template <class Model, int PREC, int SR>
 struct KernelMinBlocks {
     static constexpr bool kGeneral = Model::N == kMaxN && Model::M == kMaxM;

@@ -82,22 +82,24 @@ cudaError_t launch_rdme(const RdmeArgs &A, int family, int norm, int prec, int s
 // Threads per block of a direct-method run of n trajectories, when none is set.
 //  * Full GPU: 256 threads -- eight warps hand trajectories to each other at
 //    the end of the launch -- unless that keeps fewer than three quarters of
-//    the warps 128-thread blocks would (Schloegl uniform f16 SR, 16 of 20 warps
-//    a multiprocessor: 256 threads 40.4 against 48.1 ms at 1.5 10^5
-//    trajectories, 176.9 against 179.4 ms at 10^6).
+//    the warps 128-thread blocks would.  64 / 128 / 256 threads, ms: repressilator
+//    mixed f16 8 10^4 10.2 / 9.3 / 7.9, 3 10^5 23.0 / 23.0 / 21.5; Schloegl uniform
+//    f16 SR 8 10^4 12.3 / 11.5 / 8.9, 3 10^5 19.1 / 18.7 / 18.1; mixed bf16 within 5%.
 //  * Up to 384 lanes per multiprocessor the blocks are one wave and latency
 //    counts: the fullest multiprocessor sets the time, so the block shrinks
-//    where that spreads the lanes better (repressilator 5 10^4: 16.5 -> 14.2 ms
-//    with 128 threads; Schloegl fp64 4 10^4: 21.6 -> 17.7 ms, 10^3..2 10^4 mixed
-//    bf16 3.0 -> 2.9 ms with 64).  Above, packing is worth more (Schloegl mixed
-//    bf16 8 10^4: 4.25 ms with 256 threads, 4.33 with 128, 4.73 with 64).
+//    where that spreads the lanes better.  64 / 128 / 256 threads, ms: repressilator
+//    mixed f16 10^3 3.56 / 3.56 / 4.26, 10^4 4.14 / 4.16 / 4.92, 5 10^4 6.88 / 6.72 /
+//    7.49; Schloegl mixed bf16 10^4 2.31 / 2.33 / 2.52; fp64 10^3 10.0 / 10.3 / 13.5,
+//    2 10^4 11.4 / 13.7 / 14.5, 5 10^4 20.0 / 19.4 / 22.9.  (Where it does, it frees
+//    a sixth of those lanes or more; 2 10^4 in 32-bit modes is where the rule is
+//    off: 64 threads 3 to 5% behind 128, both ahead of 256.)
 inline int default_block(long long n, int sms, int p256, int p128)
 {
     if (n > 384ll * sms) return p256 * 8 * 4 >= p128 * 4 * 3 ? 256 : 128;
     auto fullest = [&](int b) { return ((n + b - 1) / b + sms - 1) / sms * b; };   // lanes
     int block = 256;
-    if (fullest(128) * 5 <= fullest(block) * 4) block = 128;
-    if (fullest(64) * 23 <= fullest(block) * 20) block = 64;
+    if (fullest(128) < fullest(block)) block = 128;
+    if (fullest(64) < fullest(block)) block = 64;
     return block;
 }
 

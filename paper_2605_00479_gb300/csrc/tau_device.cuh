@@ -304,8 +304,9 @@ struct Rejection {
     }
     // The binary32 test decides by hardware logarithms first.  Both sides of the
     // inequality consist of terms of size up to `size`; the contract's operations
-    // err by less than 2^-20 of it, the approximate ones (lg2.approx: 2^-22
-    // absolute in log2) by less than 2^-19, so a difference beyond 2^-17 of it
+    // err by less than 2^-20 of it, the approximate ones (lg2.approx: 2^-22 in
+    // log2, absolute for arguments in [1/2, 2] and relative elsewhere) by less
+    // than 2^-19, so a difference beyond 2^-17 of it
     // has the contract's sign.  What lies closer (0.2% of the tests at lambda =
     // 20), and lambda above 2000, where the margin would settle little, is
     // evaluated as the contract says.
