@@ -116,10 +116,10 @@ def ops_per_event(prec, rnd):
 # includes a hash of the device code, and a changed kernel reports null.
 NCU_TRAFFIC_PER_TRAJ = {
     # mixed_bf16 RN (the headline kernel), 4e5 trajectories, snapshots of X only,
-    # default launch shape, longest-first split: launch 1 13,147,648 R +
-    # 12,972,544 W; ordering kernels 10,457,344 R; launch 2 84,285,952 R +
-    # 84,645,888 W
-    ("e7dfc8f7b0080e12", "mixed_bf16:rn"): (13147648 + 12972544 + 5228800 + 8448 + 5220096 + 84285952 + 84645888)
+    # default launch shape, longest-first split: launch 1 13,324,032 R +
+    # 12,961,792 W; ordering kernels 10,456,832 R; launch 2 84,671,232 R +
+    # 85,394,176 W
+    ("db83ed165c2e6f32", "mixed_bf16:rn"): (13324032 + 12961792 + 5229056 + 8192 + 5219584 + 84671232 + 85394176)
     / 400000,
 }
 
@@ -585,23 +585,23 @@ RDME_CAP = 4_000_000
 # hash, workload, mode); a changed kernel reports null until re-counted.
 NCU_PER_UNIT = {
     # tau, 2e5 trajectories, one launch per mode (compiled Schloegl structure)
-    ("2c464a8e963606ca", "tau", "fp32:rn"): {"warp_inst": 2.8639, "dram_bytes": 0.00734},
-    ("2c464a8e963606ca", "tau", "mixed_f16:rn"): {"warp_inst": 2.9236, "dram_bytes": 0.00712},
-    ("2c464a8e963606ca", "tau", "mixed_bf16:rn"): {"warp_inst": 2.8484, "dram_bytes": 0.00725},
-    ("2c464a8e963606ca", "tau", "uniform_f16:sr"): {"warp_inst": 2.9542, "dram_bytes": 0.00747},
-    ("2c464a8e963606ca", "tau", "uniform_bf16:sr"): {"warp_inst": 2.8884, "dram_bytes": 0.00708},
+    ("4246e64760de7ca7", "tau", "fp32:rn"): {"warp_inst": 2.8697, "dram_bytes": 0.00740},
+    ("4246e64760de7ca7", "tau", "mixed_f16:rn"): {"warp_inst": 2.9294, "dram_bytes": 0.00734},
+    ("4246e64760de7ca7", "tau", "mixed_bf16:rn"): {"warp_inst": 2.8541, "dram_bytes": 0.00717},
+    ("4246e64760de7ca7", "tau", "uniform_f16:sr"): {"warp_inst": 2.9600, "dram_bytes": 0.00721},
+    ("4246e64760de7ca7", "tau", "uniform_bf16:sr"): {"warp_inst": 2.8941, "dram_bytes": 0.00706},
     # rdme, 32768 lattices, one launch per mode
-    ("24bc6759fdb0d3cf", "rdme", "fp32:rn"): {"warp_inst": 22.8227, "dram_bytes": 0.00003},
-    ("24bc6759fdb0d3cf", "rdme", "mixed_f16:rn"): {"warp_inst": 22.7984, "dram_bytes": 0.00022},
-    ("24bc6759fdb0d3cf", "rdme", "mixed_bf16:rn"): {"warp_inst": 22.8370, "dram_bytes": 0.00069},
-    ("24bc6759fdb0d3cf", "rdme", "mixed_f16:sr"): {"warp_inst": 36.5527, "dram_bytes": 0.00110},
+    ("f5bf126ba278e9f4", "rdme", "fp32:rn"): {"warp_inst": 18.8137, "dram_bytes": 0.00010},
+    ("f5bf126ba278e9f4", "rdme", "mixed_f16:rn"): {"warp_inst": 18.7738, "dram_bytes": 0.00014},
+    ("f5bf126ba278e9f4", "rdme", "mixed_bf16:rn"): {"warp_inst": 18.8059, "dram_bytes": 0.00063},
+    ("f5bf126ba278e9f4", "rdme", "mixed_f16:sr"): {"warp_inst": 35.7114, "dram_bytes": 0.00110},
 }
 
 
 def ext_source_hash(workload):
     import hashlib
     h = hashlib.sha256()
-    files = ["ssa_device.cuh", "ssa_models.h", "ssa_launch.h"]
+    files = ["ssa_device.cuh", "ssa_fast.cuh", "ssa_models.h", "ssa_launch.h"]
     files += (["tau_device.cuh", "tau_launch.h", "ssa_k_tau.cu", "ssa_k_tau_schlogl.cu"] if workload == "tau" else
               ["rdme_device.cuh", "ssa_k_rdme.cu", "ssa_k_rdme_schlogl.cu"])
     for f in files:
